@@ -22,7 +22,7 @@
 namespace sfd {
 #define SFD_DECLARE_LAUNCHER(name)                                                                   \
   cudaError_t name(const Job* d_jobs, int n_jobs, int* d_counter, int warp_floats, int warps_per_cta, \
-                   int n_ctas, int group, cudaStream_t stream);
+                   int n_ctas, int per_cta, int group, cudaStream_t stream);
 SFD_DECLARE_LAUNCHER(launch_synth_reg1)
 SFD_DECLARE_LAUNCHER(launch_synth_reg3)
 SFD_DECLARE_LAUNCHER(launch_synth_reg5)
@@ -126,17 +126,20 @@ class Pool {
 }  // namespace
 
 constexpr int kClasses = 6;   // rows per lane 1, 3, 5, 7, 9 (registers), larger (shared memory)
+// launches of a batch: each class's strings on one warp (slot = class) and
+// those on a group of warps (slot = kClasses + class)
+constexpr int kSlots = 2 * kClasses;
 
 struct sfd_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
-  cudaStream_t side[kClasses] = {};      // one per kernel class, forked from `stream`
-  cudaEvent_t fork = nullptr, join[kClasses] = {};
+  cudaStream_t side[kSlots] = {};        // one per slot, forked from `stream`
+  cudaEvent_t fork = nullptr, join[kSlots] = {};
   cudaStream_t copy = nullptr;           // host-output copies of classes already ended
   cudaEvent_t copied = nullptr;          // end of those copies, joined back to `stream`
   bool timing = false;                   // record per-class kernel times
-  cudaEvent_t t0[kClasses] = {}, t1[kClasses] = {};
-  int timed_jobs[kClasses] = {};         // jobs of each class in the last launch
+  cudaEvent_t t0[kSlots] = {}, t1[kSlots] = {};
+  int timed_jobs[kSlots] = {};           // jobs of each slot in the last launch
   Pool pool;
   int sm_count = 0;
   size_t smem_optin = 0;
@@ -144,7 +147,7 @@ struct sfd_ctx {
   int sweep_cap = 0;                       // coupled-solve sweep cap of every launch (0: kMaxSweeps)
   Job* d_jobs = nullptr;
   int job_cap = 0;
-  int* d_counter = nullptr;                // kClasses work-queue counters
+  int* d_counter = nullptr;                // work-queue counters: sm_count per slot
   int last_launches = 0;
   uint64_t h2d_bytes = 0, d2h_bytes = 0;   // all host<->device copies made
   // pinned staging of strings' initial blocks (flush_strings); the event
@@ -714,11 +717,16 @@ sfd_status ensure_jobs(sfd_ctx* c, int n) {
   return SFD_OK;
 }
 
+// Relative time of a job: steps times a fit of the measured time of a step
+// (one string per scheduler; microseconds on a GB300).
 double job_cost(const sfd_string* s, int64_t n) {
   const Desc& D = s->h;
-  double per = D.m_u * 3.0 + 40.0;
-  if (D.n_z > 0) per += 4.0 * (D.m_u + D.m_z + 40.0);
-  if (s->exc != kPluck) per *= 1.5;
+  double per = 0.4 + 0.02 * D.m_u;
+  if (!D.linear) {
+    per = 1.5 + 0.2 * D.m_u + 0.15 * D.m_z;
+    if (s->exc == kBow) per *= 1.45;
+    else if (s->exc == kHammer) per *= 1.1;
+  }
   return per * static_cast<double>(n);
 }
 
@@ -727,7 +735,17 @@ int job_class(const Desc& D) {
   return kClasses - 1;
 }
 
-using Launcher = cudaError_t (*)(const Job*, int, int*, int, int, int, int, cudaStream_t);
+// The instance of the step function a register-path string takes
+// (run_job_exc), larger for the slower ones.
+int job_variant(const Desc& D) {
+  const int z = D.m_z == 0 ? 0 : (D.z_jacobi && D.m_z <= 3 ? (D.m_z + 1) / 2 : 3);
+  return (D.exc == kBow ? 2 : D.exc == kHammer ? 1 : 0) * 8 + z * 2 + (D.linear ? 0 : 1);
+}
+
+using Launcher = cudaError_t (*)(const Job*, int, int*, int, int, int, int, int, cudaStream_t);
+// strings a CTA of each class may step at a time (the warps that the class's
+// registers allow on an SM, sfd_kernel.cu)
+const int kMaxWarps[kClasses] = {16, 8, 8, 8, 8, 4};
 const Launcher kLaunch[kClasses] = {launch_synth_reg1, launch_synth_reg3, launch_synth_reg5,
                                     launch_synth_reg7, launch_synth_reg9, launch_synth_smem};
 
@@ -736,92 +754,123 @@ const Launcher kLaunch[kClasses] = {launch_synth_reg1, launch_synth_reg3, launch
 // out), with each class's shared-memory need and the warps per CTA.
 struct Plan {
   std::vector<Job> jobs;
-  int first[kClasses + 1] = {};
-  int wf[kClasses] = {};
-  int group[kClasses] = {};  // warps per string of the class's launch (1, 2 or 4)
-  int order[kClasses] = {};  // launch order of the classes: heaviest step first
-  int wpc = 1;
+  int first[kSlots + 1] = {};
+  int wf[kSlots] = {};
+  int group[kSlots] = {};       // warps per string of the slot's launch (1, 2 or 4)
+  int regions[kSlots] = {};     // strings stepped at a time by a CTA
+  int per_cta[kSlots] = {};     // strings of a CTA's own segment of the slot's jobs
+  int ctas[kSlots] = {};
+  int order[kSlots] = {};       // launch order of the slots: heaviest step first
 };
 
 sfd_status make_plan(const sfd_ctx* c, const std::vector<Job>& jobs, const std::vector<const sfd_string*>& owners,
                      int wpc_override, Plan& P, int groups_override = -1) {
-  const int nj = static_cast<int>(jobs.size());
-  std::vector<int> order(nj), cls(nj);
+  const int nj = static_cast<int>(jobs.size()), sms = std::max(c->sm_count, 1);
+  std::vector<int> order(nj), slot(nj);
   std::vector<double> cost(nj);
   for (int i = 0; i < nj; ++i) {
     order[i] = i;
-    cls[i] = job_class(owners[i]->h);
+    slot[i] = job_class(owners[i]->h);
     cost[i] = job_cost(owners[i], jobs[i].n_samples);
   }
-  std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-    if (cls[a] != cls[b]) return cls[a] < cls[b];
-    return cost[a] > cost[b];
-  });
-  P.jobs.assign(nj, Job{});
-  for (int k = 0; k <= kClasses; ++k) P.first[k] = 0;
-  for (int k = 0; k < kClasses; ++k) P.wf[k] = 0;
-  for (int i = 0; i < nj; ++i) {
-    P.jobs[i] = jobs[order[i]];
-    P.jobs[i].sweep_cap = c->sweep_cap;
-  }
-  for (int i = 0; i < nj; ++i) {
-    const int k = cls[order[i]];
-    P.first[k + 1]++;
-    const Desc& D = owners[order[i]]->h;
-    P.wf[k] = std::max(P.wf[k], warp_smem_floats(D.m_u, D.m_z, D.z_jacobi));
-  }
-  for (int k = 0; k < kClasses; ++k) P.first[k + 1] += P.first[k];
-  for (int k = 0; k < kClasses; ++k) {
-    if (static_cast<size_t>(P.wf[k]) * sizeof(float) > c->smem_optin)
-      return fail(SFD_EINVAL, "string too large for one warp's shared memory");
-  }
-  // Classes are launched heaviest step first (shared-memory grids, then 9,
-  // 7, 5, 3, 1 rows per lane).  The block scheduler starts CTAs in launch
-  // order, and a class's persistent CTAs keep taking its jobs until its
-  // queue is empty, so when the batch does not fit on the GPU at once the
-  // class launched first holds the SMs; launched last, the slowest strings
-  // would start only when a lighter class drains and finish last (measured
-  // on the 4096-string batch: 5.3 s per step heaviest first against 6.7 s
-  // lightest first; ordering by the host's cost estimate of each class's
-  // longest job put the three 7-row strings behind the 3-row class, which
-  // alone has more CTAs than the GPU holds, and gave 6.2 s).
-  for (int k = 0; k < kClasses; ++k) P.order[k] = kClasses - 1 - k;
-  // warps per CTA: ceil(jobs / SMs), 1..4.  Warps of one CTA sit on
-  // different SM sub-partitions, so pairing jobs in a CTA keeps each string
-  // on a scheduler of its own (measured on the 256-string batch: 2 warps per
-  // CTA 27.3 M samples/s vs 19.9 M with single-warp CTAs).
-  int wpc = std::max(1, std::min(4, (nj + c->sm_count - 1) / std::max(c->sm_count, 1)));
+  int wpc = 0;   // strings per CTA asked for (0: automatic)
   if (const char* env = getenv("SFD_WARPS_PER_CTA")) {
     const int v = atoi(env);
     if (v >= 1 && v <= 4) wpc = v;
   }
   if (wpc_override >= 1 && wpc_override <= 4) wpc = wpc_override;
-  P.wpc = wpc;
-  // Warp groups: a string stepped by 2 or 4 warps of one SM (each does the
-  // transverse side, each a share of the longitudinal rows) finishes its
-  // steps sooner when its longitudinal grid is large.  Classes whose strings
-  // have such grids (folded into the sweeps; >= 3 rows per lane for pairs,
-  // >= 7 for groups of 4) get groups, heaviest class first, while the
-  // launch's warps stay within one per SM sub-partition, so groups only use
-  // schedulers that would otherwise idle.
-  for (int k = 0; k < kClasses; ++k) P.group[k] = 1;
+  // Warp groups: a string of many longitudinal rows per lane (folded into
+  // the sweeps, 5 or more) is the slowest of its launch, and stepped by 4
+  // warps of one SM (each does the transverse side, each a share of those
+  // rows) it takes 4.0 us a step instead of 6.2 (bowed, 128 x 307 intervals).
+  // The strings of most rows get a group, as many as leave the launch's
+  // other strings their warps: a group fills half an SM, a string of its own
+  // warp an eighth (a sixteenth with one transverse row per lane).
   if (groups_override < 0 ? c->warp_pairs : groups_override) {
-    int warps = nj;
-    for (int k = kClasses - 2; k >= 0; --k) {
-      const int n_k = P.first[k + 1] - P.first[k];
-      int max_mz = 0;
-      for (int i = P.first[k]; i < P.first[k + 1]; ++i) {
-        const Desc& D = owners[order[i]]->h;
-        if (D.z_jacobi) max_mz = std::max(max_mz, D.m_z);
-      }
-      if (max_mz >= 7 && warps + 3 * n_k <= 4 * c->sm_count) {
-        P.group[k] = 4;
-        warps += 3 * n_k;
-      } else if (max_mz >= 3 && warps + n_k <= 4 * c->sm_count) {
-        P.group[k] = 2;
-        warps += n_k;
-      }
+    auto rows = [&](int i) {
+      const Desc& D = owners[i]->h;
+      return slot[i] < kClasses - 1 && D.z_jacobi && D.m_z >= 5 ? D.m_z : 0;
+    };
+    double room = sms;
+    std::vector<int> heavy;
+    for (int i = 0; i < nj; ++i) {
+      room -= 1.0 / kMaxWarps[slot[i]];
+      if (rows(i) > 0) heavy.push_back(i);
     }
+    std::stable_sort(heavy.begin(), heavy.end(), [&](int x, int y) { return rows(x) > rows(y); });
+    for (int i : heavy) {
+      room -= 0.5 - 1.0 / kMaxWarps[slot[i]];
+      if (room < 0.0) break;
+      slot[i] += kClasses;
+    }
+  }
+  // within a slot, strings stepped by the same code side by side (the
+  // instances of the step function are each about as large as the
+  // instruction cache), then longest first
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+    if (slot[a] != slot[b]) return slot[a] < slot[b];
+    const int va = job_variant(owners[a]->h), vb = job_variant(owners[b]->h);
+    if (va != vb) return va > vb;
+    return cost[a] > cost[b];
+  });
+  P.jobs.assign(nj, Job{});
+  for (int k = 0; k <= kSlots; ++k) P.first[k] = 0;
+  for (int k = 0; k < kSlots; ++k) P.wf[k] = 0;
+  for (int i = 0; i < nj; ++i) {
+    P.jobs[i] = jobs[order[i]];
+    P.jobs[i].sweep_cap = c->sweep_cap;
+    const int k = slot[order[i]];
+    P.first[k + 1]++;
+    const Desc& D = owners[order[i]]->h;
+    P.wf[k] = std::max(P.wf[k], warp_smem_floats(D.m_u, D.m_z, D.z_jacobi));
+  }
+  for (int k = 0; k < kSlots; ++k) P.first[k + 1] += P.first[k];
+  for (int k = 0; k < kSlots; ++k) {
+    if (static_cast<size_t>(P.wf[k]) * sizeof(float) > c->smem_optin)
+      return fail(SFD_EINVAL, "string too large for one warp's shared memory");
+  }
+  // Slots are launched heaviest step first (groups, then shared-memory grids,
+  // then 9, 7, 5, 3, 1 rows per lane).  The block scheduler starts CTAs in
+  // launch order, and a class's CTAs keep taking its jobs until none is left,
+  // so when the batch does not fit on the GPU at once the class launched
+  // first holds the SMs; launched last, the slowest strings would start only
+  // when a lighter class drains and finish last (measured on the 4096-string
+  // batch: 5.3 s per step heaviest first against 6.7 s lightest first;
+  // ordering by the host's cost estimate of each class's longest job put the
+  // three 7-row strings behind the 3-row class, which alone has more CTAs
+  // than the GPU holds, and gave 6.2 s).
+  for (int k = 0; k < kSlots; ++k) P.order[k] = kSlots - 1 - k;
+  // CTAs: every class gets its share of the SMs by cost, one CTA on each,
+  // and every CTA a segment of the class's jobs (sorted: the warps of an SM
+  // then run the same instance of the step function and share it in the
+  // instruction cache).  A segment of up to kMaxWarps strings is stepped at
+  // once, a longer one in rounds; CTAs that run out take from the others.
+  const int n_groups = P.first[kSlots] - P.first[kClasses], n_own = nj - n_groups;
+  const int own_sms = std::max(1, sms - (n_groups + 1) / 2);
+  double w_all = 0, w[kSlots] = {};
+  for (int i = 0; i < nj; ++i) {
+    w[slot[i]] += cost[i];
+    if (slot[i] < kClasses) w_all += cost[i];
+  }
+  for (int k = 0; k < kSlots; ++k) {
+    const int n_k = P.first[k + 1] - P.first[k], cls = k % kClasses;
+    P.group[k] = k >= kClasses ? 4 : 1;
+    if (n_k == 0) continue;
+    const size_t wbytes = static_cast<size_t>(P.wf[k]) * sizeof(float);
+    const int most = static_cast<int>(std::max<size_t>(1, std::min<size_t>(
+        k >= kClasses ? 1 : (wpc ? 4 : kMaxWarps[cls]), c->smem_optin / wbytes)));
+    if (k >= kClasses) {
+      P.regions[k] = P.per_cta[k] = 1;
+    } else if (wpc) {   // as asked
+      P.regions[k] = P.per_cta[k] = std::min(most, wpc);
+    } else {
+      int share = n_own <= own_sms ? n_k : static_cast<int>(own_sms * (w[k] / std::max(w_all, 1e-300)));
+      share = std::max(1, std::min(share, n_k));
+      P.per_cta[k] = (n_k + share - 1) / share;
+      const int rounds = (P.per_cta[k] + most - 1) / most;
+      P.regions[k] = (P.per_cta[k] + rounds - 1) / rounds;
+    }
+    P.ctas[k] = (n_k + P.per_cta[k] - 1) / P.per_cta[k];
   }
   return SFD_OK;
 }
@@ -833,29 +882,22 @@ sfd_status make_plan(const sfd_ctx* c, const std::vector<Job>& jobs, const std::
 sfd_status issue_plan(sfd_ctx* c, const Plan& P, const Job* d_jobs) {
   c->last_launches = 0;
   int active = 0;
-  for (int k = 0; k < kClasses; ++k) active += P.first[k + 1] > P.first[k];
+  for (int k = 0; k < kSlots; ++k) active += P.first[k + 1] > P.first[k];
   if (active == 0) return SFD_OK;
   if (active > 1) SFD_CUDA(cudaEventRecord(c->fork, c->stream));
-  for (int k = 0; k < kClasses; ++k) c->timed_jobs[k] = 0;
-  for (int kk = 0; kk < kClasses; ++kk) {
+  for (int k = 0; k < kSlots; ++k) c->timed_jobs[k] = 0;
+  for (int kk = 0; kk < kSlots; ++kk) {
     const int k = P.order[kk];
     const int n_k = P.first[k + 1] - P.first[k];
     if (n_k == 0) continue;
-    const size_t wbytes = static_cast<size_t>(P.wf[k]) * sizeof(float);
-    // strings (regions) per CTA, limited by shared memory; a group of warps
-    // per string (at most 4 warps per CTA)
-    const int g = P.group[k];
-    int regions = static_cast<int>(std::min<size_t>(static_cast<size_t>(P.wpc), c->smem_optin / wbytes));
-    regions = std::max(1, std::min(regions, 4 / g));
-    const int wpc = regions * g;
-    const int n_ctas = (n_k + regions - 1) / regions;
     cudaStream_t st = c->stream;
     if (active > 1) {
       st = c->side[k];
       SFD_CUDA(cudaStreamWaitEvent(st, c->fork, 0));
     }
     if (c->timing) SFD_CUDA(cudaEventRecord(c->t0[k], st));
-    cudaError_t e = kLaunch[k](d_jobs + P.first[k], n_k, c->d_counter + k, P.wf[k], wpc, n_ctas, P.group[k], st);
+    cudaError_t e = kLaunch[k % kClasses](d_jobs + P.first[k], n_k, c->d_counter + k * c->sm_count, P.wf[k],
+                               P.regions[k] * P.group[k], P.ctas[k], P.per_cta[k], P.group[k], st);
     if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
     if (c->timing) {
       SFD_CUDA(cudaEventRecord(c->t1[k], st));
@@ -895,9 +937,9 @@ sfd_status launch_jobs(sfd_ctx* c, std::vector<Job>& jobs, const std::vector<con
 // copies after it there.
 sfd_status copy_out_by_class(sfd_ctx* c, const Plan& P, const float* dout, float* out_host) {
   int active = 0;
-  for (int k = 0; k < kClasses; ++k) active += P.first[k + 1] > P.first[k];
+  for (int k = 0; k < kSlots; ++k) active += P.first[k + 1] > P.first[k];
   const cudaStream_t st = active > 1 ? c->copy : c->stream;
-  for (int kk = 0; kk < kClasses; ++kk) {
+  for (int kk = 0; kk < kSlots; ++kk) {
     const int k = P.order[kk];
     if (P.first[k + 1] == P.first[k]) continue;
     if (active > 1) SFD_CUDA(cudaStreamWaitEvent(st, c->join[k], 0));
@@ -1016,7 +1058,7 @@ sfd_status sfd_ctx_create(int device, void* cuda_stream, size_t mem_budget_bytes
   c->smem_optin = prop.sharedMemPerBlockOptin - kStaticSmemBytes;
   sfd_status rc = c->pool.init(mem_budget_bytes ? mem_budget_bytes : (size_t{256} << 20));
   if (rc) { delete c; return rc; }
-  if ((e = cudaMalloc(&c->d_counter, sizeof(int) * kClasses)) != cudaSuccess) {
+  if ((e = cudaMalloc(&c->d_counter, sizeof(int) * kSlots * c->sm_count)) != cudaSuccess) {
     c->pool.release();
     delete c;
     return cuda_fail(e, "cudaMalloc(counter)");
@@ -1024,7 +1066,7 @@ sfd_status sfd_ctx_create(int device, void* cuda_stream, size_t mem_budget_bytes
   bool ok = cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) == cudaSuccess &&
             cudaEventCreateWithFlags(&c->copied, cudaEventDisableTiming) == cudaSuccess &&
             cudaStreamCreateWithFlags(&c->copy, cudaStreamNonBlocking) == cudaSuccess;
-  for (int k = 0; k < kClasses && ok; ++k) {
+  for (int k = 0; k < kSlots && ok; ++k) {
     ok = cudaStreamCreateWithFlags(&c->side[k], cudaStreamNonBlocking) == cudaSuccess &&
          cudaEventCreateWithFlags(&c->join[k], cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreate(&c->t0[k]) == cudaSuccess && cudaEventCreate(&c->t1[k]) == cudaSuccess;
@@ -1041,7 +1083,7 @@ void sfd_ctx_destroy(sfd_ctx* c) {
   if (!c) return;
   cudaSetDevice(c->device);
   cudaStreamSynchronize(c->stream);
-  for (int k = 0; k < kClasses; ++k) {
+  for (int k = 0; k < kSlots; ++k) {
     if (c->side[k]) cudaStreamDestroy(c->side[k]);
     if (c->join[k]) cudaEventDestroy(c->join[k]);
     if (c->t0[k]) cudaEventDestroy(c->t0[k]);
@@ -1113,12 +1155,14 @@ sfd_status sfd_ctx_kernel_times(sfd_ctx* c, float* ms, int32_t* n_jobs) {
   if (!c || !ms || !n_jobs) return fail(SFD_EINVAL, "NULL argument");
   sfd_status rc = set_device(c);
   if (rc) return rc;
-  for (int k = 0; k < kClasses; ++k) {
-    ms[k] = 0.f;
-    n_jobs[k] = c->timing ? c->timed_jobs[k] : 0;
-    if (n_jobs[k] == 0) continue;
+  for (int k = 0; k < kClasses; ++k) ms[k] = 0.f, n_jobs[k] = 0;
+  for (int k = 0; c->timing && k < kSlots; ++k) {   // a class's launches run side by side: the longer one
+    if (c->timed_jobs[k] == 0) continue;
+    float t = 0.f;
     SFD_CUDA(cudaEventSynchronize(c->t1[k]));
-    SFD_CUDA(cudaEventElapsedTime(&ms[k], c->t0[k], c->t1[k]));
+    SFD_CUDA(cudaEventElapsedTime(&t, c->t0[k], c->t1[k]));
+    ms[k % kClasses] = std::max(ms[k % kClasses], t);
+    n_jobs[k % kClasses] += c->timed_jobs[k];
   }
   return SFD_OK;
 }
@@ -1801,7 +1845,7 @@ sfd_status sfd_batch_autotune(sfd_batch* b, int64_t probe_samples, int32_t* best
   cudaEventCreate(&e1);
   float best_ms = 0.f;
   int best = 0, best_groups = 0;
-  const int candidates[3] = {1, 2, 4};
+  const int candidates[4] = {1, 2, 4, 0};   // 0: automatic (reported as 4)
   // warp groups are a candidate only if they would form for this batch
   bool groups_form = false;
   {
@@ -1809,10 +1853,11 @@ sfd_status sfd_batch_autotune(sfd_batch* b, int64_t probe_samples, int32_t* best
     std::vector<const sfd_string*> owners(b->strings.begin(), b->strings.end());
     Plan P;
     if (make_plan(c, jobs, owners, 0, P, 1) == SFD_OK)
-      for (int k = 0; k < kClasses; ++k) groups_form = groups_form || P.group[k] > 1;
+      groups_form = P.first[kSlots] > P.first[kClasses];
   }
-  for (int cj = 0; cj < 6 && rc == SFD_OK; ++cj) {
-    const int ci = cj % 3, groups = cj / 3;   // warps per CTA x warp groups off / on
+  int best_wpc = 0;
+  for (int cj = 0; cj < 8 && rc == SFD_OK; ++cj) {
+    const int ci = cj % 4, groups = cj / 4;   // warps per CTA x warp groups off / on
     if (groups && !groups_form) continue;
     // fresh clones of the current state for every candidate
     std::vector<sfd_string*> cl;
@@ -1839,7 +1884,12 @@ sfd_status sfd_batch_autotune(sfd_batch* b, int64_t probe_samples, int32_t* best
         float ms = 0.f;
         if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
         if (e != cudaSuccess) rc = cuda_fail(e, "autotune timing");
-        else if (best == 0 || ms < best_ms) { best_ms = ms; best = candidates[ci]; best_groups = groups; }
+        else if (best == 0 || ms < best_ms) {
+          best_ms = ms;
+          best_wpc = candidates[ci];
+          best = best_wpc ? best_wpc : 4;
+          best_groups = groups;
+        }
       }
     }
     cudaStreamSynchronize(c->stream);
@@ -1849,7 +1899,7 @@ sfd_status sfd_batch_autotune(sfd_batch* b, int64_t probe_samples, int32_t* best
   cudaEventDestroy(e1);
   c->pool.dealloc(dout);
   if (rc) return rc;
-  b->wpc = best;
+  b->wpc = best_wpc;
   b->groups = best_groups;
   if (best_warps_per_cta) *best_warps_per_cta = best;
   return SFD_OK;
@@ -2009,7 +2059,7 @@ extern "C" sfd_status sfd_synthesize_noalloc(int device, void* cuda_stream, cons
   const int k = job_class(D);
   int* counter = reinterpret_cast<int*>(b + o_cnt) + k;   // the launcher clears it on `stream`
   e = kLaunch[k](reinterpret_cast<const Job*>(b + o_job), 1, counter,
-                 warp_smem_floats(D.m_u, D.m_z, D.z_jacobi), 1, 1, 1, stream);
+                 warp_smem_floats(D.m_u, D.m_z, D.z_jacobi), 1, 1, 1, 1, stream);
   if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
   e = cudaMemcpyAsync(&sc, b + o_sc, sizeof(Scalars), cudaMemcpyDeviceToHost, stream);
   if (e != cudaSuccess) return cuda_fail(e, "status read");

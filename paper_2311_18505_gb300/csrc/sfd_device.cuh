@@ -14,6 +14,21 @@ namespace sfd {
 
 #define SFD_FULL 0xffffffffu
 
+// a compile-time flag passed to a generic lambda
+template <bool B>
+struct BoolC {
+  static constexpr bool value = B;
+};
+
+// The same pointer, opaque to the compiler: what is read through it is read
+// where it stands (from L1) rather than hoisted out of the time loop into a
+// register that then lives for the whole note.
+template <class T>
+__device__ __forceinline__ const T* reread(const T* p) {
+  asm volatile("" : "+l"(p));
+  return p;
+}
+
 // whole-warp shuffles by precision (the templated solvers below; df64 in
 // sfd_df64.cuh)
 __device__ __forceinline__ float shfl_up(float v, int s) { return __shfl_up_sync(SFD_FULL, v, s); }
@@ -211,10 +226,9 @@ __device__ __forceinline__ float zinterp(const float* __restrict__ A, int node, 
 // fractional part (exact for any n, and no FP64 arithmetic, which runs at a
 // small fraction of the FP32 rate on this GPU, enters the step); glissando:
 // 2^{2 D min(n k, T) / T}, i.e. held at 2^{2D} from step n_end on.
-__device__ __forceinline__ float mod_factor(int kind, uint64_t inc_fx, uint64_t phase_fx, float depth2,
-                                            float inc, float hold, int64_t n_end, int64_t n) {
+__device__ __forceinline__ float mod_factor_at(int kind, uint64_t t_fx, float depth2, float inc, float hold,
+                                               int64_t n_end, int64_t n) {   // t_fx: the vibrato's phase at n
   if (kind == 1) {
-    const uint64_t t_fx = static_cast<uint64_t>(n) * inc_fx + phase_fx;
     const float t = static_cast<float>(static_cast<uint32_t>(t_fx >> 40)) * 5.9604644775390625e-8f;   // 2^-24
     // sin(2 pi t) = -sin(2 pi (t - 1/2)), whose argument lies in [-pi, pi):
     // there the hardware sine's absolute error is ~2^-21, i.e. ~1e-8 in rm
@@ -222,6 +236,10 @@ __device__ __forceinline__ float mod_factor(int kind, uint64_t inc_fx, uint64_t 
   }
   if (kind == 2) return exp2f(n < n_end ? inc * static_cast<float>(n) : hold);
   return 1.f;
+}
+__device__ __forceinline__ float mod_factor(int kind, uint64_t inc_fx, uint64_t phase_fx, float depth2,
+                                            float inc, float hold, int64_t n_end, int64_t n) {
+  return mod_factor_at(kind, static_cast<uint64_t>(n) * inc_fx + phase_fx, depth2, inc, hold, n_end, n);
 }
 
 // Bow controls of step n from the descriptor's breakpoint envelopes

@@ -46,26 +46,45 @@
 
 namespace sfd {
 
-// One resident block of up to 4 warps per SM lets each class use up to 255
-// registers.  Capping them at 168 or 128 (3 or 4 resident blocks) makes ptxas
-// spill 0.1-3 KB per thread and, measured on the 4096-string modulated
-// batch, lowers throughput from 124 M to 92 M / 88 M samples/s despite the
-// extra warps.
+// Warps per CTA, one CTA per SM.  One row per lane fits 128 registers with
+// little spilling, so 16 warps of it share an SM: 2432 equal strings take
+// 2.4 us a step (plucked) and 3.5 us (bowed), against 3.9 and 5.4 us in two
+// rounds of 8 warps at 255 registers.  Three rows per lane spill 200 bytes in
+// the bowed instances at 168 registers (12 warps) and took 3.6 us a step
+// instead of 2.9, more than the extra warps gain (4096-string batch 10.5 ms
+// per 512 samples against 10.2), so they and the larger classes keep 8 warps.
+#ifdef SFD_MU
+constexpr int kMaxThreads = kWarp * (SFD_MU == 1 ? 16 : 8);
+#else
+constexpr int kMaxThreads = kWarp * 4;
+#endif
+
+// Which warp takes which string.  The host sorts a class's jobs by the
+// instance of the step function they take and gives CTA c the segment
+// [c per_cta, (c + 1) per_cta) of them; the CTA's `regions` warps start on
+// the segment's first jobs and take the others as they finish, by a counter
+// per segment, then those of segments still waiting.  So the warps of an SM
+// step strings of one or two kinds: each instance's time loop is 10-25 KB of
+// code, and with the kinds mixed on every SM (one queue for all CTAs) their
+// instruction fetches missed the cache: 1000 mixed strings then took 14.3 us
+// a step, in segments 8.8 us (one generic loop for every kind: 10.0 us).
 //
-// With group = 2 or 4 (register path only) the CTA's warps work in groups
-// (warps g*group .. g*group + group - 1 share region g): the group's first
-// warp takes the next job from the queue and passes it on through shared
-// memory (named barrier 1 + g over the whole group), and the warps the job
-// can use step it (run_job_reg, in-job barrier 1 + g for pairs, 3 for
-// groups of 4, whose unused warps meanwhile wait at barrier 1).  The job
-// index cells alternate so that a cell is rewritten only after every warp
-// of the group has passed the next barrier, i.e. after all have read it.
-__global__ void __launch_bounds__(128, 1) SFD_KERNEL(const Job* __restrict__ jobs, int n_jobs,
-                                                    int* __restrict__ counter, int warp_floats, int group) {
+// With group = 2 or 4 (register path only, at most 4 warps per CTA; the
+// host launches groups of 4) the
+// CTA's warps work in groups (warps g*group .. g*group + group - 1 share
+// region g): the group's first warp takes the next job and passes it on
+// through shared memory (named barrier 1 + g over the whole group), and the
+// warps the job can use step it (run_job_reg, in-job barrier 1 + g for
+// pairs, 3 for groups of 4, whose unused warps meanwhile wait at barrier 1).
+// The job index cells alternate so that a cell is rewritten only after every
+// warp of the group has passed the next barrier, i.e. after all have read it.
+__global__ void __launch_bounds__(kMaxThreads, 1) SFD_KERNEL(const Job* __restrict__ jobs, int n_jobs,
+                                                             int* __restrict__ counters, int warp_floats,
+                                                             int per_cta, int group) {
   extern __shared__ float smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & (kWarp - 1);
 #ifdef SFD_MU
-  __shared__ float xcells[2][1024];  // per group: [buffer][warp][chg, mag, chx, mgx][lane]
+  __shared__ __align__(16) float xcells[2][1024];  // per group: [buffer][warp][chg, mag, chx, mgx][lane]
   __shared__ int jcell[2][2];        // per group: job index, alternating
   const int npw = group == 4 ? 4 : (group == 2 ? 2 : 1);
 #else
@@ -73,14 +92,46 @@ __global__ void __launch_bounds__(128, 1) SFD_KERNEL(const Job* __restrict__ job
   (void)group;
 #endif
   const int pi = warp / npw, pw = warp - pi * npw;
-  float* wbase = smem + static_cast<size_t>(pi) * warp_floats;
+  const int regions = (blockDim.x >> 5) / npw;
+  const int region = pi * warp_floats;
+  const int n_ctas = gridDim.x;
+  // the next job of segment v, or n_jobs; its first `regions` are taken as
+  // the CTA starts, the others in the order of the segment's counter
+  auto segment_end = [&](int v) { return min((v + 1) * per_cta, n_jobs); };
+  auto take = [&](int v) {
+    const int j = v * per_cta + regions + atomicAdd(&counters[v], 1);
+    return j < segment_end(v) ? j : n_jobs;
+  };
+  auto next_job = [&](bool first) {
+    if (first) {
+      const int j = blockIdx.x * per_cta + pi;
+      return j < segment_end(blockIdx.x) ? j : n_jobs;
+    }
+    if (per_cta <= regions) return n_jobs;   // every job began as its CTA started
+    int j = n_jobs;
+    if (lane == 0) j = take(blockIdx.x);
+    j = __shfl_sync(SFD_FULL, j, 0);
+    // this segment is empty: help the others, from the next one on
+    for (int b = 0; j >= n_jobs && b < n_ctas; b += kWarp) {
+      const int o = b + lane, v = o < n_ctas ? (blockIdx.x + 1 + o) % n_ctas : 0;
+      const int seen = o < n_ctas ? *const_cast<volatile int*>(&counters[v]) : 0;
+      unsigned left = __ballot_sync(SFD_FULL, o < n_ctas && v * per_cta + regions + seen < segment_end(v));
+      while (left && j >= n_jobs) {
+        const int src = __ffs(left) - 1;
+        left &= left - 1;
+        const int vv = __shfl_sync(SFD_FULL, v, src);
+        if (lane == 0) j = take(vv);
+        j = __shfl_sync(SFD_FULL, j, 0);
+      }
+    }
+    return j;
+  };
 #ifdef SFD_MU
   int it = 0;
 #endif
-  for (;;) {
-    int j = 0;
-    if (lane == 0 && pw == 0) j = atomicAdd(counter, 1);
-    j = __shfl_sync(SFD_FULL, j, 0);
+  for (bool first = true;; first = false) {
+    int j = n_jobs;
+    if (pw == 0) j = next_job(first);
 #ifdef SFD_MU
     if (npw > 1) {
       if (pw == 0 && lane == 0) jcell[pi][it & 1] = j;
@@ -91,9 +142,9 @@ __global__ void __launch_bounds__(128, 1) SFD_KERNEL(const Job* __restrict__ job
 #endif
     if (j >= n_jobs) break;
 #ifdef SFD_MU
-    run_job_reg<SFD_MU>(jobs[j], wbase, lane, pw, npw, npw == 4 ? 3 : 1 + pi, npw > 1 ? xcells[pi] : nullptr);
+    run_job_reg<SFD_MU>(jobs[j], region, lane, pw, npw, npw == 4 ? 3 : 1 + pi, npw > 1 ? xcells[pi] : nullptr);
 #else
-    run_job(jobs[j], wbase, lane);
+    run_job(jobs[j], smem + region, lane);
 #endif
   }
 }
@@ -129,25 +180,32 @@ cudaError_t raise_smem_limit() {
 }
 }  // namespace
 
-// Host-side launcher of this class (C++ linkage, called by sfd_api.cu).  The
-// job counter is cleared on the same stream before the kernel starts.  With
-// group = 2 or 4 (register classes; warps_per_cta a multiple of it, 4 for
-// groups of 4) each string gets a group of warps and one shared-memory
-// region per group.
-cudaError_t SFD_LAUNCHER(const Job* d_jobs, int n_jobs, int* d_counter, int warp_floats, int warps_per_cta,
-                         int n_ctas, int group, cudaStream_t stream) {
+// Host-side launcher of this class (C++ linkage, called by sfd_api.cu): CTA
+// c steps jobs [c per_cta, (c + 1) per_cta), warps_per_cta / group of them at
+// a time.  Segments longer than that use one counter per CTA, cleared on the
+// same stream before the kernel starts (d_counters holds n_ctas then).  With
+// group = 2 or 4 (register classes; at most 4 warps per CTA, a multiple of
+// it) each string gets a group of warps and one shared-memory region per
+// group.
+cudaError_t SFD_LAUNCHER(const Job* d_jobs, int n_jobs, int* d_counters, int warp_floats, int warps_per_cta,
+                         int n_ctas, int per_cta, int group, cudaStream_t stream) {
 #ifndef SFD_MU
   group = 1;
 #endif
   if (group != 1 && group != 2 && group != 4) return cudaErrorInvalidValue;
-  if (warps_per_cta % group != 0 || (group == 4 && warps_per_cta != 4)) return cudaErrorInvalidValue;
+  if (warps_per_cta < 1 || warps_per_cta * kWarp > kMaxThreads || warps_per_cta % group != 0 ||
+      (group > 1 && warps_per_cta > 4))
+    return cudaErrorInvalidValue;
   const int regions = warps_per_cta / group;
   const size_t smem = static_cast<size_t>(warp_floats) * regions * sizeof(float);
   cudaError_t e = raise_smem_limit();
   if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(d_counter, 0, sizeof(int), stream);
-  if (e != cudaSuccess) return e;
-  SFD_KERNEL<<<n_ctas, warps_per_cta * kWarp, smem, stream>>>(d_jobs, n_jobs, d_counter, warp_floats, group);
+  if (per_cta > regions) {
+    e = cudaMemsetAsync(d_counters, 0, sizeof(int) * n_ctas, stream);
+    if (e != cudaSuccess) return e;
+  }
+  SFD_KERNEL<<<n_ctas, warps_per_cta * kWarp, smem, stream>>>(d_jobs, n_jobs, d_counters, warp_floats, per_cta,
+                                                              group);
   return cudaGetLastError();
 }
 
