@@ -14,6 +14,8 @@
 namespace sfd {
 cudaError_t launch_adjoint(const AdjJob* d_jobs, int n_jobs, int smem_bytes, cudaStream_t stream);
 cudaError_t adjoint_static_smem(size_t* bytes);
+cudaError_t launch_adjoint_rows(const AdjJob* d_jobs, int n_jobs, int threads, int smem_bytes, cudaStream_t stream);
+cudaError_t adjoint_rows_static_smem(size_t* bytes);
 }
 
 namespace {
@@ -38,6 +40,9 @@ struct sfd_tape {
   size_t traj_stride = 0;               // floats per string in the replay record
   size_t adj_stride = 0;                // doubles per string of adjoint state
   int adj_smem = 0;                     // shared-memory bytes of the adjoint kernel
+  // strings of the one-thread-per-row adjoint kernel come first in the job table
+  std::vector<int> adj_order;
+  int n_rows = 0, rows_threads = 0, rows_smem = 0;
   char* d_ckpt = nullptr;
   float* d_traj = nullptr;
   double* d_adj = nullptr;
@@ -142,12 +147,33 @@ sfd_status sfd_tape_create(sfd_ctx* c, int32_t n, const sfd_string_params* param
     t->ckpt_stride = std::max(t->ckpt_stride, round_up(t->st_bytes.back(), kTapeAlign));
     t->traj_stride = std::max(t->traj_stride, static_cast<size_t>(t->rec_stride.back()) * t->K);
     t->adj_stride = std::max(t->adj_stride, round_up(2 * D.n_u + 4 * D.n_z + 2, 64));
-    t->adj_smem = std::max(t->adj_smem, adj_smem_bytes(D.m_u, D.m_z));
   }
-  size_t adj_static = 0;
+  size_t adj_static = 0, rows_static = 0;
   if (rc == SFD_OK) {
-    const cudaError_t e = adjoint_static_smem(&adj_static);
+    cudaError_t e = adjoint_static_smem(&adj_static);
+    if (e == cudaSuccess) e = adjoint_rows_static_smem(&rows_static);
     if (e != cudaSuccess) rc = cuda_fail(e, "adjoint kernel attributes");
+  }
+  // Which adjoint kernel: one thread per row wherever the grid allows it (at
+  // most 255 transverse rows, longitudinal off-diagonal folded into the
+  // sweeps: its chain is shorter at every size: 20 us a step against 41 on 64 strings
+  // of 40-1000 Hz, 15 against 26 on one of 31 x 4 rows); larger or strongly damped grids take four warps per string.
+  if (rc == SFD_OK) {
+    std::vector<int> rest;
+    for (int i = 0; i < n; ++i) {
+      const Desc& D = t->fw[i]->h;
+      const int bytes = adj_rows_smem_bytes(D.n_u, D.n_z);
+      if (D.n_u <= kAdjRowsMax && (D.n_z == 0 || D.z_jacobi) && bytes + rows_static <= c->smem_optin) {
+        t->adj_order.push_back(i);
+        t->rows_threads = std::max(t->rows_threads, (D.n_u + 1 + kWarp - 1) / kWarp * kWarp);
+        t->rows_smem = std::max(t->rows_smem, bytes);
+      } else {
+        rest.push_back(i);
+        t->adj_smem = std::max(t->adj_smem, adj_smem_bytes(D.m_u, D.m_z));
+      }
+    }
+    t->n_rows = static_cast<int>(t->adj_order.size());
+    t->adj_order.insert(t->adj_order.end(), rest.begin(), rest.end());
   }
   if (rc == SFD_OK && static_cast<size_t>(t->adj_smem) + adj_static > c->smem_optin)
     rc = fail(SFD_EINVAL, "a string's grid exceeds the adjoint kernel's shared memory");
@@ -270,14 +296,15 @@ sfd_status sfd_tape_backward(sfd_tape* t, const float* dy_device, double* grad) 
     }
     if (!t->d_traj_full && (rc = launch_jobs(c, jobs, owners))) return rc;
     // reverse sweep over the segment's levels (m0, m1]
-    for (int i = 0; i < t->n; ++i) {
+    for (int q = 0; q < t->n; ++q) {
+      const int i = t->adj_order[q];
       const sfd_string* s = t->rp[i];
       const Desc& D = s->h;
       char* slot = ckpt_slot(t, i, seg);
       auto at = [&](const void* dev) {
         return reinterpret_cast<const float*>(slot + (static_cast<const char*>(dev) - s->block - t->st_off[i]));
       };
-      AdjJob& a = aj[i];
+      AdjJob& a = aj[q];
       a.desc = s->d_desc;
       a.u0 = at(D.u);
       a.du0 = at(D.du);
@@ -295,7 +322,9 @@ sfd_status sfd_tape_backward(sfd_tape* t, const float* dy_device, double* grad) 
       a.pluck_pos = s->exc == kPluck ? static_cast<float>(s->pluck_pos) : -1.f;
     }
     SFD_CUDA(h2d(c, t->d_ajobs, aj.data(), sizeof(AdjJob) * t->n));
-    SFD_CUDA(launch_adjoint(t->d_ajobs, t->n, t->adj_smem, c->stream));
+    SFD_CUDA(launch_adjoint_rows(t->d_ajobs, t->n_rows, t->rows_threads, t->rows_smem, c->stream));
+    if (t->n_rows < t->n)
+      SFD_CUDA(launch_adjoint(t->d_ajobs + t->n_rows, t->n - t->n_rows, t->adj_smem, c->stream));
     // (the next segment's replay and job table follow in stream order)
   }
   std::vector<double> g(static_cast<size_t>(t->n) * kGradSlots);

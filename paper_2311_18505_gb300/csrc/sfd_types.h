@@ -153,4 +153,18 @@ inline __host__ __device__ int adj_smem_bytes(int m_u, int m_z) {
   return (17 * 8 + 9 * 4) * ru + (13 * 8 + 6 * 4) * rz;
 }
 
+// The adjoint sweep with one thread per transverse row (sfd_adjoint_rows.cu):
+// up to kAdjRowsMax rows, a folded longitudinal matrix (or none), whose
+// coupling vanishes within kAdjRowsZLev reduction levels.  Shared memory:
+// three trajectory records, 14 double-float arrays and the reduction weights
+// (two per level) per transverse row, 18 double-float arrays per longitudinal
+// one, a float array of each and an int array.
+constexpr int kAdjRowsMax = 255;
+constexpr int kAdjRowsLev = 8;    // reduction levels of up to 256 rows
+constexpr int kAdjRowsZLev = 3;
+inline __host__ __device__ int adj_rows_smem_bytes(int n_u, int n_z) {
+  const int rec = (2 * n_u + 2 * n_z + 2 + 3) & ~3, ru = n_u + 4, rz = n_z > 0 ? n_z + 4 : 0;
+  return 4 * (3 * rec + 28 * ru + 4 * kAdjRowsLev * n_u + 36 * rz + ru + 2 * rz);
+}
+
 }  // namespace sfd
