@@ -22,7 +22,7 @@
 namespace sfd {
 #define SFD_DECLARE_LAUNCHER(name)                                                                   \
   cudaError_t name(const Job* d_jobs, int n_jobs, int* d_counter, int warp_floats, int warps_per_cta, \
-                   int n_ctas, int per_cta, int group, cudaStream_t stream);
+                   int n_ctas, int queued, int group, cudaStream_t stream);
 SFD_DECLARE_LAUNCHER(launch_synth_reg1)
 SFD_DECLARE_LAUNCHER(launch_synth_reg3)
 SFD_DECLARE_LAUNCHER(launch_synth_reg5)
@@ -718,14 +718,18 @@ sfd_status ensure_jobs(sfd_ctx* c, int n) {
 }
 
 // Relative time of a job: steps times a fit of the measured time of a step
-// (one string per scheduler; microseconds on a GB300).
+// (alone on a scheduler, microseconds on a GB300; plucked and struck strings
+// 1.9-2.5, bowed 2.7-3.3 with up to 3 longitudinal rows per lane, 4.3-10 with
+// 5-25).
 double job_cost(const sfd_string* s, int64_t n) {
   const Desc& D = s->h;
-  double per = 0.4 + 0.02 * D.m_u;
+  double per = 0.4 + 0.01 * D.m_u;
   if (!D.linear) {
-    per = 1.5 + 0.2 * D.m_u + 0.15 * D.m_z;
-    if (s->exc == kBow) per *= 1.45;
-    else if (s->exc == kHammer) per *= 1.1;
+    per = D.m_u == 1 ? 1.9 : 1.1 + 0.25 * D.m_u;
+    double z = D.m_z >= 5 || (D.m_z > 0 && !D.z_jacobi) ? 0.33 + 0.115 * D.m_z : 0.05 * D.m_z;
+    if (s->exc == kBow) per *= 1.42, z *= 1.8;
+    per += z;
+    if (D.m_u > kMaxRegRows) per *= 3.0;   // shared-memory path
   }
   return per * static_cast<double>(n);
 }
@@ -758,7 +762,7 @@ struct Plan {
   int wf[kSlots] = {};
   int group[kSlots] = {};       // warps per string of the slot's launch (1, 2 or 4)
   int regions[kSlots] = {};     // strings stepped at a time by a CTA
-  int per_cta[kSlots] = {};     // strings of a CTA's own segment of the slot's jobs
+  int queued[kSlots] = {};      // some segment is longer than that
   int ctas[kSlots] = {};
   int order[kSlots] = {};       // launch order of the slots: heaviest step first
 };
@@ -841,36 +845,59 @@ sfd_status make_plan(const sfd_ctx* c, const std::vector<Job>& jobs, const std::
   // than the GPU holds, and gave 6.2 s).
   for (int k = 0; k < kSlots; ++k) P.order[k] = kSlots - 1 - k;
   // CTAs: every class gets its share of the SMs by cost, one CTA on each,
-  // and every CTA a segment of the class's jobs (sorted: the warps of an SM
+  // and every CTA a segment of about equal cost of the class's jobs (sorted: the warps of an SM
   // then run the same instance of the step function and share it in the
   // instruction cache).  A segment of up to kMaxWarps strings is stepped at
   // once, a longer one in rounds; CTAs that run out take from the others.
   const int n_groups = P.first[kSlots] - P.first[kClasses], n_own = nj - n_groups;
   const int own_sms = std::max(1, sms - (n_groups + 1) / 2);
-  double w_all = 0, w[kSlots] = {};
+  double w_all = 0, w[kSlots] = {};   // SM time: a string holds 1 / kMaxWarps of one
   for (int i = 0; i < nj; ++i) {
-    w[slot[i]] += cost[i];
-    if (slot[i] < kClasses) w_all += cost[i];
+    const int k = slot[i];
+    w[k] += cost[i] / kMaxWarps[k % kClasses];
+    if (k < kClasses) w_all += cost[i] / kMaxWarps[k];
   }
   for (int k = 0; k < kSlots; ++k) {
     const int n_k = P.first[k + 1] - P.first[k], cls = k % kClasses;
     P.group[k] = k >= kClasses ? 4 : 1;
     if (n_k == 0) continue;
+    Job* const J = &P.jobs[P.first[k]];
     const size_t wbytes = static_cast<size_t>(P.wf[k]) * sizeof(float);
     const int most = static_cast<int>(std::max<size_t>(1, std::min<size_t>(
-        k >= kClasses ? 1 : (wpc ? 4 : kMaxWarps[cls]), c->smem_optin / wbytes)));
-    if (k >= kClasses) {
-      P.regions[k] = P.per_cta[k] = 1;
-    } else if (wpc) {   // as asked
-      P.regions[k] = P.per_cta[k] = std::min(most, wpc);
+        k >= kClasses ? 1 : (wpc ? wpc : kMaxWarps[cls]), c->smem_optin / wbytes)));
+    int longest = 1;
+    P.ctas[k] = 0;
+    if (k >= kClasses || wpc) {   // groups, or as asked
+      longest = most;
+      for (int j = 0; j < n_k; j += most) J[P.ctas[k]++].seg = j;
     } else {
       int share = n_own <= own_sms ? n_k : static_cast<int>(own_sms * (w[k] / std::max(w_all, 1e-300)));
       share = std::max(1, std::min(share, n_k));
-      P.per_cta[k] = (n_k + share - 1) / share;
-      const int rounds = (P.per_cta[k] + most - 1) / most;
-      P.regions[k] = (P.per_cta[k] + rounds - 1) / rounds;
+      // segments of equal cost, of no more strings than the fewest rounds hold
+      const int per_cta = (n_k + share - 1) / share, rounds = (per_cta + most - 1) / most;
+      double left = 0;
+      for (int j = 0; j < n_k; ++j) left += cost[order[P.first[k] + j]];
+      for (int j = 0; j < n_k;) {
+        const double part = left / std::max(1, std::min(share - P.ctas[k], n_k - j));
+        const int begin = j;
+        double sum = 0;
+        while (j < n_k && j - begin < rounds * most) {
+          const double cj = cost[order[P.first[k] + j]];
+          if (j > begin && sum + 0.5 * cj > part) break;
+          sum += cj;
+          ++j;
+        }
+        left -= sum;
+        longest = std::max(longest, j - begin);
+        if (P.ctas[k] == c->sm_count) {   // (no more counters: the last segment takes the rest)
+          longest = std::max(longest, n_k - J[P.ctas[k] - 1].seg);
+          break;
+        }
+        J[P.ctas[k]++].seg = begin;
+      }
     }
-    P.ctas[k] = (n_k + P.per_cta[k] - 1) / P.per_cta[k];
+    P.regions[k] = std::min(most, longest);
+    P.queued[k] = longest > P.regions[k];
   }
   return SFD_OK;
 }
@@ -897,7 +924,7 @@ sfd_status issue_plan(sfd_ctx* c, const Plan& P, const Job* d_jobs) {
     }
     if (c->timing) SFD_CUDA(cudaEventRecord(c->t0[k], st));
     cudaError_t e = kLaunch[k % kClasses](d_jobs + P.first[k], n_k, c->d_counter + k * c->sm_count, P.wf[k],
-                               P.regions[k] * P.group[k], P.ctas[k], P.per_cta[k], P.group[k], st);
+                               P.regions[k] * P.group[k], P.ctas[k], P.queued[k], P.group[k], st);
     if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
     if (c->timing) {
       SFD_CUDA(cudaEventRecord(c->t1[k], st));
@@ -2059,7 +2086,7 @@ extern "C" sfd_status sfd_synthesize_noalloc(int device, void* cuda_stream, cons
   const int k = job_class(D);
   int* counter = reinterpret_cast<int*>(b + o_cnt) + k;   // the launcher clears it on `stream`
   e = kLaunch[k](reinterpret_cast<const Job*>(b + o_job), 1, counter,
-                 warp_smem_floats(D.m_u, D.m_z, D.z_jacobi), 1, 1, 1, 1, stream);
+                 warp_smem_floats(D.m_u, D.m_z, D.z_jacobi), 1, 1, 0, 1, stream);
   if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
   e = cudaMemcpyAsync(&sc, b + o_sc, sizeof(Scalars), cudaMemcpyDeviceToHost, stream);
   if (e != cudaSuccess) return cuda_fail(e, "status read");

@@ -60,8 +60,8 @@ constexpr int kMaxThreads = kWarp * 4;
 #endif
 
 // Which warp takes which string.  The host sorts a class's jobs by the
-// instance of the step function they take and gives CTA c the segment
-// [c per_cta, (c + 1) per_cta) of them; the CTA's `regions` warps start on
+// instance of the step function they take and gives every CTA a segment of
+// them of about equal cost (Job::seg); the CTA's `regions` warps start on
 // the segment's first jobs and take the others as they finish, by a counter
 // per segment, then those of segments still waiting.  So the warps of an SM
 // step strings of one or two kinds: each instance's time loop is 10-25 KB of
@@ -80,7 +80,7 @@ constexpr int kMaxThreads = kWarp * 4;
 // warp of the group has passed the next barrier, i.e. after all have read it.
 __global__ void __launch_bounds__(kMaxThreads, 1) SFD_KERNEL(const Job* __restrict__ jobs, int n_jobs,
                                                              int* __restrict__ counters, int warp_floats,
-                                                             int per_cta, int group) {
+                                                             int queued, int group) {
   extern __shared__ float smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & (kWarp - 1);
 #ifdef SFD_MU
@@ -97,17 +97,15 @@ __global__ void __launch_bounds__(kMaxThreads, 1) SFD_KERNEL(const Job* __restri
   const int n_ctas = gridDim.x;
   // the next job of segment v, or n_jobs; its first `regions` are taken as
   // the CTA starts, the others in the order of the segment's counter
-  auto segment_end = [&](int v) { return min((v + 1) * per_cta, n_jobs); };
+  auto segment = [&](int v) { return v < n_ctas ? jobs[v].seg : n_jobs; };
+  const int seg0 = segment(blockIdx.x), seg1 = segment(blockIdx.x + 1);
   auto take = [&](int v) {
-    const int j = v * per_cta + regions + atomicAdd(&counters[v], 1);
-    return j < segment_end(v) ? j : n_jobs;
+    const int j = segment(v) + regions + atomicAdd(&counters[v], 1);
+    return j < segment(v + 1) ? j : n_jobs;
   };
   auto next_job = [&](bool first) {
-    if (first) {
-      const int j = blockIdx.x * per_cta + pi;
-      return j < segment_end(blockIdx.x) ? j : n_jobs;
-    }
-    if (per_cta <= regions) return n_jobs;   // every job began as its CTA started
+    if (first) return seg0 + pi < seg1 ? seg0 + pi : n_jobs;
+    if (!queued) return n_jobs;   // every job began as its CTA started
     int j = n_jobs;
     if (lane == 0) j = take(blockIdx.x);
     j = __shfl_sync(SFD_FULL, j, 0);
@@ -115,7 +113,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) SFD_KERNEL(const Job* __restri
     for (int b = 0; j >= n_jobs && b < n_ctas; b += kWarp) {
       const int o = b + lane, v = o < n_ctas ? (blockIdx.x + 1 + o) % n_ctas : 0;
       const int seen = o < n_ctas ? *const_cast<volatile int*>(&counters[v]) : 0;
-      unsigned left = __ballot_sync(SFD_FULL, o < n_ctas && v * per_cta + regions + seen < segment_end(v));
+      unsigned left = __ballot_sync(SFD_FULL, o < n_ctas && segment(v) + regions + seen < segment(v + 1));
       while (left && j >= n_jobs) {
         const int src = __ffs(left) - 1;
         left &= left - 1;
@@ -181,14 +179,14 @@ cudaError_t raise_smem_limit() {
 }  // namespace
 
 // Host-side launcher of this class (C++ linkage, called by sfd_api.cu): CTA
-// c steps jobs [c per_cta, (c + 1) per_cta), warps_per_cta / group of them at
-// a time.  Segments longer than that use one counter per CTA, cleared on the
-// same stream before the kernel starts (d_counters holds n_ctas then).  With
+// c steps its segment of the jobs, warps_per_cta / group of them at a time.
+// With `queued` (some segment is longer than that) the CTAs take them by one
+// counter each, cleared on the same stream before the kernel starts.  With
 // group = 2 or 4 (register classes; at most 4 warps per CTA, a multiple of
 // it) each string gets a group of warps and one shared-memory region per
 // group.
 cudaError_t SFD_LAUNCHER(const Job* d_jobs, int n_jobs, int* d_counters, int warp_floats, int warps_per_cta,
-                         int n_ctas, int per_cta, int group, cudaStream_t stream) {
+                         int n_ctas, int queued, int group, cudaStream_t stream) {
 #ifndef SFD_MU
   group = 1;
 #endif
@@ -200,11 +198,11 @@ cudaError_t SFD_LAUNCHER(const Job* d_jobs, int n_jobs, int* d_counters, int war
   const size_t smem = static_cast<size_t>(warp_floats) * regions * sizeof(float);
   cudaError_t e = raise_smem_limit();
   if (e != cudaSuccess) return e;
-  if (per_cta > regions) {
+  if (queued) {
     e = cudaMemsetAsync(d_counters, 0, sizeof(int) * n_ctas, stream);
     if (e != cudaSuccess) return e;
   }
-  SFD_KERNEL<<<n_ctas, warps_per_cta * kWarp, smem, stream>>>(d_jobs, n_jobs, d_counters, warp_floats, per_cta,
+  SFD_KERNEL<<<n_ctas, warps_per_cta * kWarp, smem, stream>>>(d_jobs, n_jobs, d_counters, warp_floats, queued,
                                                               group);
   return cudaGetLastError();
 }

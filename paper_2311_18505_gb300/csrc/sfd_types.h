@@ -105,7 +105,7 @@ struct Job {
   float* traj;
   int64_t traj_stride;
   int32_t sweep_cap;      // largest Gauss-Seidel sweep count per step (0: kMaxSweeps)
-  int32_t pad_;
+  int32_t seg;            // entry c of a launch's jobs: where CTA c's segment of them begins
 };
 
 // One string's part of a reverse sweep of the discrete adjoint over the
