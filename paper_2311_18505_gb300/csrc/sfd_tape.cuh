@@ -256,12 +256,10 @@ sfd_status sfd_tape_forward(sfd_tape* t, float* y_device) {
   }
   SFD_CUDA(cudaStreamSynchronize(c->stream));
   int worst = SFD_OK;
-  for (sfd_string* s : t->fw) {
-    Scalars sc{};
-    if ((rc = read_status(s, &sc))) return rc;
-    const sfd_status st = status_code(sc);
+  std::vector<int32_t> codes(t->n);
+  if ((rc = read_statuses(c, owners.data(), owners.size(), codes.data()))) return rc;
+  for (int32_t st : codes)
     if (st == SFD_EUNSTABLE || (st == SFD_ENOCONV && worst == SFD_OK)) worst = st;
-  }
   t->forward_done = true;
   if (worst == SFD_EUNSTABLE) return fail(worst, "a string's state became non-finite");
   if (worst == SFD_ENOCONV) return fail(worst, "a coupled solve reached its sweep cap (result kept)");
