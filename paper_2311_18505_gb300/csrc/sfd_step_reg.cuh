@@ -136,6 +136,7 @@ __device__ __forceinline__ float node_interp(const float (&x)[MU], NodePos a, No
 // values: its coupling A (C) to that side is exactly zero by then, since row
 // 0 has no sub-diagonal and the last row no super-diagonal, so no select is
 // needed.  The reciprocal of each pivot is taken once, before the shuffles.
+// On entry rd.nlev is the last step's number of reduction levels (a guess).
 template <int MU>
 __device__ __forceinline__ void tri_factor_r(const float (&sb)[MU], float (&iv)[MU], float (&cp)[MU],
                                              float (&ff)[MU], float (&gg)[MU], Red& rd) {
@@ -169,26 +170,37 @@ __device__ __forceinline__ void tri_factor_r(const float (&sb)[MU], float (&iv)[
     g0n = __shfl_down_sync(SFD_FULL, gg[0], 1);
   }
   const float cl = cp[MU - 1];   // (lane 31's is a pad row's: zero)
-  float A = al[MU - 1], B = fmaf(cl, g0n, 1.f), C = cl * f0n;
+  const float A0 = al[MU - 1], B0 = fmaf(cl, g0n, 1.f), C0 = cl * f0n;
   rd.cl = cl;
-  rd.nlev = 5;
+  // The reduction stops at the first level whose couplings have all dropped
+  // below kPcrDrop (at most 5).  That level hardly changes from step to step,
+  // so the levels of the last step are run without looking, and two votes
+  // tell whether it was the first: not dropped one level before, dropped at
+  // it.  (A vote and a branch at every level cost some 45 cycles each on the
+  // step's chain.)
+  for (;;) {
+    float A = A0, B = B0, C = C0;
+    bool before = false;    // dropped one level before the last
 #pragma unroll
-  for (int l = 0; l < 5; ++l) { rd.k1[l] = 0.f; rd.k2[l] = 0.f; }
-#pragma unroll
-  for (int l = 0; l < 5; ++l) {
-    if (__all_sync(SFD_FULL, fabsf(A) + fabsf(C) <= kPcrDrop * fabsf(B))) { rd.nlev = l; break; }
-    const int s = 1 << l;
-    const float rB = fast_rcp(B);
-    const float Am = __shfl_up_sync(SFD_FULL, A, s), Cm = __shfl_up_sync(SFD_FULL, C, s);
-    const float Ap = __shfl_down_sync(SFD_FULL, A, s), Cp = __shfl_down_sync(SFD_FULL, C, s);
-    const float k1 = A * __shfl_up_sync(SFD_FULL, rB, s), k2 = C * __shfl_down_sync(SFD_FULL, rB, s);
-    A = -Am * k1;
-    C = -Cp * k2;
-    B = fmaf(-Ap, k2, fmaf(-Cm, k1, B));
-    rd.k1[l] = k1;
-    rd.k2[l] = k2;
+    for (int l = 0; l < 5; ++l) {
+      if (l >= rd.nlev) break;
+      before = fabsf(A) + fabsf(C) <= kPcrDrop * fabsf(B);
+      const int s = 1 << l;
+      const float rB = fast_rcp(B);
+      const float Am = __shfl_up_sync(SFD_FULL, A, s), Cm = __shfl_up_sync(SFD_FULL, C, s);
+      const float Ap = __shfl_down_sync(SFD_FULL, A, s), Cp = __shfl_down_sync(SFD_FULL, C, s);
+      const float k1 = A * __shfl_up_sync(SFD_FULL, rB, s), k2 = C * __shfl_down_sync(SFD_FULL, rB, s);
+      A = -Am * k1;
+      C = -Cp * k2;
+      B = fmaf(-Ap, k2, fmaf(-Cm, k1, B));
+      rd.k1[l] = k1;
+      rd.k2[l] = k2;
+    }
+    rd.binv = fast_rcp(B);
+    if (__all_sync(SFD_FULL, before) && rd.nlev > 0) --rd.nlev;
+    else if (rd.nlev < 5 && !__all_sync(SFD_FULL, fabsf(A) + fabsf(C) <= kPcrDrop * fabsf(B))) ++rd.nlev;
+    else break;
   }
-  rd.binv = fast_rcp(B);
 }
 
 // Solve one (NR = 1) or two (NR = 2) right-hand sides in place, interleaved.
@@ -597,6 +609,9 @@ __device__ __noinline__ void step_string(const Job& job, int region, int lane, c
 
   // ---- constant matrices ----
   Red rdu, rdz;
+  rdu.nlev = 3;
+#pragma unroll
+  for (int l = 0; l < 5; ++l) { rdu.k1[l] = 0.f; rdu.k2[l] = 0.f; }
   const float dz_diag = 1.f + Dp->s0 + 2.f * s1l;
   const float dz_inv = fast_rcp(dz_diag);
   if (kFact) {
@@ -763,24 +778,44 @@ __device__ __noinline__ void step_string(const Job& job, int region, int lane, c
     const bool need_resp = !LIN && ((EXC == kHammer && k2G > 0.f) || (EXC == kBow && FB > 0.f));
 
     // ---- stage 1: transverse right-hand side and matrix (registers) ----
-    float Ue[MU + 4], DUe[MU + 2], GL[MU], GR[MU];
+    float Ue[MU + 4], DUe[MU + 2], GL[MU], GR[MU], gi[MU + 1], yi[MU + 1], gi2[MU + 1];
     extend<MU>(U, Ue, lane);
     extend1<MU>(DU, DUe, lane);
 #pragma unroll
+    for (int r = 0; r < MU + 1; ++r) gi[r] = Ue[r + 2] - Ue[r + 1];   // interval left of row r
+#pragma unroll
     for (int r = 0; r < MU; ++r) {   // interval differences; zero on pad rows
       const bool real = ub + r < n_u;
-      GL[r] = real ? Ue[r + 2] - Ue[r + 1] : 0.f;
-      GR[r] = real ? Ue[r + 3] - Ue[r + 2] : 0.f;
+      GL[r] = real ? gi[r] : 0.f;
+      GR[r] = real ? gi[r + 1] : 0.f;
     }
     float ZTe[MU + 2];
     if (kHasZ) interp_z(Z, oZ, ZTe);
+    // the strain's and the coupling's terms of every interval (each serves the
+    // rows on both sides)
+    if (!LIN) {
+#pragma unroll
+      for (int r = 0; r < MU + 1; ++r) {
+        const float gk = gi[r];
+        gi2[r] = __fmul_rn(gk, gk);
+        yi[r] = __fmul_rn(2.f * ca * gi2[r], gk);
+        if (kHasZ) {
+          const float zk = ZTe[r + 1] - ZTe[r];
+          // (the two forms differ in the last bit; each class keeps the one
+          // its samples have had)
+          if (MU >= 5) yi[r] = fmaf(2.f * ca * gi2[r], gk, __fmul_rn(4.f * cb * gk, zk));
+          else yi[r] = fmaf(4.f * cb * gk, zk, yi[r]);
+        }
+      }
+    }
     float RA[MU], fv[MU];
 #pragma unroll
     for (int r = 0; r < MU; ++r) {
       const int i = ub + r;
+      const bool real = i < n_u;
       fv[r] = 0.f;
       const float u0 = Ue[r + 2], um1 = Ue[r + 1], up1 = Ue[r + 3], um2 = Ue[r], up2 = Ue[r + 4];
-      const float gl = GL[r], gr = GR[r];
+      const float gl = gi[r], gr = gi[r + 1];
       const float d2 = gr - gl;
       float d4 = ((up2 - up1) - gr) - 2.f * d2 + (gl - (um1 - um2));
       if (i == 0) d4 += bsgn * u0;
@@ -789,26 +824,12 @@ __device__ __noinline__ void step_string(const Job& job, int region, int lane, c
       const float d2du = (DUe[r + 2] - du0) - (du0 - DUe[r]);
       float rhs = fmaf(2.f * s1, d2du, fmaf(-2.f * s0u, du0, fmaf(-mu2, d4, fmaf(lam2, d2, __fmul_rn(lam2_lo, d2)))));
       if (!LIN) {
-        const float gl2 = __fmul_rn(gl, gl), gr2 = __fmul_rn(gr, gr);
-        float yl = __fmul_rn(2.f * ca * gl2, gl), yr = __fmul_rn(2.f * ca * gr2, gr);
-        if (kHasZ) {
-          const float zl = ZTe[r + 1] - ZTe[r], zg = ZTe[r + 2] - ZTe[r + 1];
-          // (the two forms differ in the last bit; each class keeps the one its
-          // samples have had)
-          if (MU >= 5) {
-            yl = fmaf(2.f * ca * gl2, gl, __fmul_rn(4.f * cb * gl, zl));
-            yr = fmaf(2.f * ca * gr2, gr, __fmul_rn(4.f * cb * gr, zg));
-          } else {
-            yl = fmaf(4.f * cb * gl, zl, yl);
-            yr = fmaf(4.f * cb * gr, zg, yr);
-          }
-          fv[r] = gr2 - gl2;   // zero on pad rows
-        }
-        rhs = __fadd_rn(rhs, __fsub_rn(yr, yl));
-        const bool real = i < n_u;
-        SB[r] = (real && i > 0) ? fmaf(-ca, gl2, og) : 0.f;
-        IV[r] = real ? fmaf(ca, __fadd_rn(gl2, gr2), dg) : 1.f;
-        CPr[r] = i < n_u - 1 ? fmaf(-ca, gr2, og) : 0.f;
+        // (fv of a pad row goes to no slot)
+        if (kHasZ) fv[r] = gi2[r + 1] - gi2[r];
+        rhs = __fadd_rn(rhs, __fsub_rn(yi[r + 1], yi[r]));
+        SB[r] = (real && i > 0) ? fmaf(-ca, gi2[r], og) : 0.f;
+        IV[r] = real ? fmaf(ca, __fadd_rn(gi2[r], gi2[r + 1]), dg) : 1.f;
+        CPr[r] = i < n_u - 1 ? fmaf(-ca, gi2[r + 1], og) : 0.f;
         DG0[r] = IV[r];
         CP0[r] = CPr[r];
       }
