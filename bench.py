@@ -398,6 +398,7 @@ def run_ours(args, ws, rank, local):
         free_batch(hb)
     # timed: inputs for every step created (and captured) before the region
     batches = [prepared_batch() for _ in range(args.steps)]
+    graph_launches = sfd.sfd_last_launch_count(ctx)   # the kernels of one captured step
     torch.cuda.synchronize(dev)
     ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(args.steps)]
     class_ms = [0.0] * sfd.SFD_KERNEL_CLASSES
@@ -417,7 +418,7 @@ def run_ours(args, ws, rank, local):
             # together and the GPU's dispatch order varies (4.5-5.5 s per
             # step on the 4096-string batch against 4.51-4.55 s this way)
             ev[i][1].synchronize()
-        launches += len(set(classes)) if g is not None else sfd.sfd_last_launch_count(ctx)
+        launches += graph_launches if g is not None else sfd.sfd_last_launch_count(ctx)
         if g is None:
             # per-class kernel times, recorded with events on each kernel's own stream
             ms_k, _ = sfd.sfd_ctx_kernel_times(ctx)

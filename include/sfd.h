@@ -265,13 +265,14 @@ int32_t sfd_last_launch_count(const sfd_ctx* ctx);
 
 /* Number of step-kernel classes: strings are grouped by transverse rows per
  * lane (1, 3, 5, 7, 9 held in registers; more in shared memory) and each
- * group runs as its own persistent kernel, concurrently with the others. */
+ * class runs as its own persistent kernels (its strings of few longitudinal
+ * rows, of many, and of warp groups apart), all concurrently. */
 #define SFD_KERNEL_CLASSES 6
 
 /* Per-class kernel timing: when enabled, every launch records CUDA events
- * around each class kernel on the stream it runs on; sfd_ctx_kernel_times
+ * around each class's kernels on the streams they run on; sfd_ctx_kernel_times
  * waits for them and reports, for the last batch/synthesize call, each
- * class's kernel time [ms] and job count (ms[SFD_KERNEL_CLASSES],
+ * class's longest kernel time [ms] and its job count (ms[SFD_KERNEL_CLASSES],
  * n_jobs[SFD_KERNEL_CLASSES]; zeros for classes not launched). */
 sfd_status sfd_ctx_set_timing(sfd_ctx* ctx, int32_t enable);
 sfd_status sfd_ctx_kernel_times(sfd_ctx* ctx, float* ms, int32_t* n_jobs);
@@ -281,10 +282,10 @@ sfd_status sfd_ctx_kernel_times(sfd_ctx* ctx, float* ms, int32_t* n_jobs);
  * the GPU has warp schedulers leaves schedulers idle and its time is that of
  * its slowest string.  With groups enabled, strings whose longitudinal grid
  * is large (the longitudinal coupling folded into the Gauss-Seidel sweeps;
- * 3 or more longitudinal rows per lane for 2 warps, 7 or more for 4) are
- * each stepped by 2 or 4 warps of one SM, which split the longitudinal
- * rows, as long as the launch then still has at most one warp per
- * scheduler.  The samples are bit for bit the same with and without groups.
+ * 5 or more longitudinal rows per lane) are each stepped by 4 warps of one
+ * SM (8 with 13 to 24 rows per lane), which split the longitudinal rows:
+ * those of most rows first, as many as leave the launch's other strings
+ * their warps.  The samples are bit for bit the same with and without groups.
  * enable = 0 steps every string with one warp. */
 sfd_status sfd_ctx_set_warp_pairs(sfd_ctx* ctx, int32_t enable);
 
@@ -304,9 +305,9 @@ sfd_status sfd_string_kernel_class(const sfd_string* s, int32_t* cls);
  * kernels wrote straight into pinned host memory count as device->host). */
 sfd_status sfd_ctx_transfer_bytes(const sfd_ctx* ctx, uint64_t* h2d_total, uint64_t* d2h_total);
 
-/* Warps per CTA for this batch's launches: 1..4, or 0 (default) for
- * automatic (jobs / SMs, clamped).  Warps of one CTA run on different SM
- * sub-partitions, so this sets how many strings share an SM. */
+/* Warps per CTA for this batch's launches: 1..3 as asked; 0 (default) or 4,
+ * the largest, for the library's own packing (one CTA per SM of up to 16
+ * strings of one kind, CTAs divided among the classes by cost). */
 sfd_status sfd_batch_set_warps_per_cta(sfd_batch* b, int32_t warps_per_cta);
 
 /* Choose warps per CTA and warp groups by measurement: runs probe_samples

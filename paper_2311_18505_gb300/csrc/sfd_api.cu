@@ -23,7 +23,7 @@
 namespace sfd {
 #define SFD_DECLARE_LAUNCHER(name)                                                                   \
   cudaError_t name(const Job* d_jobs, int n_jobs, int* d_counter, int warp_floats, int warps_per_cta, \
-                   int n_ctas, int queued, int group, cudaStream_t stream);
+                   int n_ctas, int queued, int group, int smem_least, cudaStream_t stream);
 SFD_DECLARE_LAUNCHER(launch_synth_reg1)
 SFD_DECLARE_LAUNCHER(launch_synth_reg3)
 SFD_DECLARE_LAUNCHER(launch_synth_reg5)
@@ -127,14 +127,16 @@ class Pool {
 }  // namespace
 
 constexpr int kClasses = 6;   // rows per lane 1, 3, 5, 7, 9 (registers), larger (shared memory)
-// launches of a batch: each class's strings on one warp (slot = class) and
-// those on a group of warps (slot = kClasses + class)
-constexpr int kSlots = 2 * kClasses;
+// launches of a batch (slot = class + kClasses x kind): each class's strings
+// of few longitudinal rows per lane, those of many on a warp of their own,
+// those on a group of 4 and of 8 warps
+enum SlotKind { kFew = 0, kMany = 1, kGroup4 = 2, kGroup8 = 3, kSlotKinds = 4 };
+constexpr int kSlots = kSlotKinds * kClasses;
 
 struct sfd_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
-  cudaStream_t side[kSlots] = {};        // one per slot, forked from `stream`
+  cudaStream_t side[kSlots] = {};        // one per slot in use (ensure_slots), forked from `stream`
   cudaEvent_t fork = nullptr, join[kSlots] = {};
   cudaStream_t copy = nullptr;           // host-output copies of classes already ended
   cudaEvent_t copied = nullptr;          // end of those copies, joined back to `stream`
@@ -747,10 +749,14 @@ int job_variant(const Desc& D) {
   return (D.exc == kBow ? 2 : D.exc == kHammer ? 1 : 0) * 8 + z * 2 + (D.linear ? 0 : 1);
 }
 
-using Launcher = cudaError_t (*)(const Job*, int, int*, int, int, int, int, int, cudaStream_t);
+using Launcher = cudaError_t (*)(const Job*, int, int*, int, int, int, int, int, int, cudaStream_t);
 // strings a CTA of each class may step at a time (the warps that the class's
 // registers allow on an SM, sfd_kernel.cu)
 const int kMaxWarps[kClasses] = {16, 8, 8, 8, 8, 4};
+// longitudinal rows per lane of which a group has 8 warps, three in the
+// registers of each: 5.3-5.5 us a step, in groups of 4 6.1-6.3 (bowed, 17 and
+// 19 rows; from 29 rows on, more warps gain nothing)
+constexpr int kWideRows = 13, kWideMost = 24;
 const Launcher kLaunch[kClasses] = {launch_synth_reg1, launch_synth_reg3, launch_synth_reg5,
                                     launch_synth_reg7, launch_synth_reg9, launch_synth_smem};
 
@@ -766,9 +772,25 @@ struct Plan {
   int queued[kSlots] = {};      // some segment is longer than that
   int ctas[kSlots] = {};
   int order[kSlots] = {};       // launch order of the slots: heaviest step first
+  int smem_least = 0;           // shared memory a CTA asks for at least (no two on an SM)
 };
 
-sfd_status make_plan(const sfd_ctx* c, const std::vector<Job>& jobs, const std::vector<const sfd_string*>& owners,
+// The side stream and events of every slot the plan uses, made on the slot's
+// first use (planning, never launching: a launch may be captured).
+sfd_status ensure_slots(sfd_ctx* c, const Plan& P) {
+  for (int k = 0; k < kSlots; ++k) {
+    if (P.first[k + 1] == P.first[k] || c->join[k]) continue;
+    cudaEvent_t j = nullptr;
+    if (!c->side[k]) SFD_CUDA(cudaStreamCreateWithFlags(&c->side[k], cudaStreamNonBlocking));
+    if (!c->t0[k]) SFD_CUDA(cudaEventCreate(&c->t0[k]));
+    if (!c->t1[k]) SFD_CUDA(cudaEventCreate(&c->t1[k]));
+    SFD_CUDA(cudaEventCreateWithFlags(&j, cudaEventDisableTiming));
+    c->join[k] = j;
+  }
+  return SFD_OK;
+}
+
+sfd_status make_plan(sfd_ctx* c, const std::vector<Job>& jobs, const std::vector<const sfd_string*>& owners,
                      int wpc_override, Plan& P, int groups_override = -1) {
   const int nj = static_cast<int>(jobs.size()), sms = std::max(c->sm_count, 1);
   std::vector<int> order(nj), slot(nj);
@@ -778,35 +800,40 @@ sfd_status make_plan(const sfd_ctx* c, const std::vector<Job>& jobs, const std::
     slot[i] = job_class(owners[i]->h);
     cost[i] = job_cost(owners[i], jobs[i].n_samples);
   }
-  int wpc = 0;   // strings per CTA asked for (0: automatic)
+  int wpc = 0;   // strings per CTA asked for (0 or 4: automatic)
   if (const char* env = getenv("SFD_WARPS_PER_CTA")) {
     const int v = atoi(env);
     if (v >= 1 && v <= 4) wpc = v;
   }
   if (wpc_override >= 1 && wpc_override <= 4) wpc = wpc_override;
-  // Warp groups: a string of many longitudinal rows per lane (folded into
-  // the sweeps, 5 or more) is the slowest of its launch, and stepped by 4
-  // warps of one SM (each does the transverse side, each a share of those
-  // rows) it takes 4.0 us a step instead of 6.2 (bowed, 128 x 307 intervals).
-  // The strings of most rows get a group, as many as leave the launch's
-  // other strings their warps: a group fills half an SM, a string of its own
-  // warp an eighth (a sixteenth with one transverse row per lane).
+  if (wpc == 4) wpc = 0;   // the largest: as many as the class's registers allow
+  // Strings of many longitudinal rows per lane are launched apart: their
+  // shared-memory region would leave room for fewer of the others on an SM.
+  for (int i = 0; i < nj; ++i)
+    if (slot[i] < kClasses - 1 && (owners[i]->h.m_z >= 5 || (owners[i]->h.m_z > 0 && !owners[i]->h.z_jacobi)))
+      slot[i] += kMany * kClasses;
+  // Warp groups: such a string (the matrix folded into the sweeps) is the
+  // slowest of its launch; stepped by 4 or 8 warps of one SM (each does the
+  // transverse side, each a share of those rows) it takes 4.0 us a step
+  // instead of 6.2 (bowed, 128 x 307 intervals, 4 warps).  The strings of
+  // most rows get a group, as many as leave the launch's other strings their
+  // warps: a group of 4 fills half an SM, a string of its own warp an eighth
+  // (a sixteenth with one transverse row per lane).
   if (groups_override < 0 ? c->warp_pairs : groups_override) {
-    auto rows = [&](int i) {
-      const Desc& D = owners[i]->h;
-      return slot[i] < kClasses - 1 && D.z_jacobi && D.m_z >= 5 ? D.m_z : 0;
-    };
-    double room = sms;
+    double room = sms - kClasses;   // (every class may leave a CTA partly filled)
     std::vector<int> heavy;
     for (int i = 0; i < nj; ++i) {
-      room -= 1.0 / kMaxWarps[slot[i]];
-      if (rows(i) > 0) heavy.push_back(i);
+      room -= 1.0 / kMaxWarps[slot[i] % kClasses];
+      if (slot[i] >= kClasses && owners[i]->h.z_jacobi) heavy.push_back(i);
     }
-    std::stable_sort(heavy.begin(), heavy.end(), [&](int x, int y) { return rows(x) > rows(y); });
+    std::stable_sort(heavy.begin(), heavy.end(),
+                     [&](int x, int y) { return owners[x]->h.m_z > owners[y]->h.m_z; });
     for (int i : heavy) {
-      room -= 0.5 - 1.0 / kMaxWarps[slot[i]];
+      const int m_z = owners[i]->h.m_z;
+      const bool wide = m_z >= kWideRows && m_z <= kWideMost;
+      room -= (wide ? 1.0 : 0.5) - 1.0 / kMaxWarps[slot[i] % kClasses];
       if (room < 0.0) break;
-      slot[i] += kClasses;
+      slot[i] += ((wide ? kGroup8 : kGroup4) - kMany) * kClasses;
     }
   }
   // within a slot, strings stepped by the same code side by side (the
@@ -834,8 +861,8 @@ sfd_status make_plan(const sfd_ctx* c, const std::vector<Job>& jobs, const std::
     if (static_cast<size_t>(P.wf[k]) * sizeof(float) > c->smem_optin)
       return fail(SFD_EINVAL, "string too large for one warp's shared memory");
   }
-  // Slots are launched heaviest step first (groups, then shared-memory grids,
-  // then 9, 7, 5, 3, 1 rows per lane).  The block scheduler starts CTAs in
+  // Slots are launched heaviest step first (groups, then many longitudinal
+  // rows, then shared-memory grids and 9, 7, 5, 3, 1 transverse rows per lane).  The block scheduler starts CTAs in
   // launch order, and a class's CTAs keep taking its jobs until none is left,
   // so when the batch does not fit on the GPU at once the class launched
   // first holds the SMs; launched last, the slowest strings would start only
@@ -844,47 +871,80 @@ sfd_status make_plan(const sfd_ctx* c, const std::vector<Job>& jobs, const std::
   // ordering by the host's cost estimate of each class's longest job put the
   // three 7-row strings behind the 3-row class, which alone has more CTAs
   // than the GPU holds, and gave 6.2 s).
-  for (int k = 0; k < kSlots; ++k) P.order[k] = kSlots - 1 - k;
+  for (int k = 0; k < kSlots; ++k) P.order[k] = kSlots - 1 - k, P.ctas[k] = 0;
   // CTAs: every class gets its share of the SMs by cost, one CTA on each,
   // and every CTA a segment of about equal cost of the class's jobs (sorted: the warps of an SM
   // then run the same instance of the step function and share it in the
   // instruction cache).  A segment of up to kMaxWarps strings is stepped at
   // once, a longer one in rounds; CTAs that run out take from the others.
-  const int n_groups = P.first[kSlots] - P.first[kClasses], n_own = nj - n_groups;
-  const int own_sms = std::max(1, sms - (n_groups + 1) / 2);
+  const int n4 = P.first[kGroup8 * kClasses] - P.first[kGroup4 * kClasses];
+  const int n8 = P.first[kSlots] - P.first[kGroup8 * kClasses];
+  constexpr int kOwn = kGroup4 * kClasses;   // slots below: a warp per string
   double w_all = 0, w[kSlots] = {};   // SM time: a string holds 1 / kMaxWarps of one
+  double top[kSlots] = {};            // the slot's longest job
   for (int i = 0; i < nj; ++i) {
     const int k = slot[i];
     w[k] += cost[i] / kMaxWarps[k % kClasses];
-    if (k < kClasses) w_all += cost[i] / kMaxWarps[k];
+    top[k] = std::max(top[k], cost[i]);
+    if (k < kOwn) w_all += cost[i] / kMaxWarps[k % kClasses];
+  }
+  // SMs per slot: when one round holds every string, at least what that
+  // takes, the others to whichever slot would end last; else by cost
+  int most_k[kSlots] = {}, share_k[kSlots] = {}, least = 0;
+  for (int k = 0; k < kSlots; ++k) {
+    const int n_k = P.first[k + 1] - P.first[k];
+    if (n_k == 0) continue;
+    const size_t wbytes = static_cast<size_t>(P.wf[k]) * sizeof(float);
+    most_k[k] = static_cast<int>(std::max<size_t>(1, std::min<size_t>(
+        k >= kOwn ? 1 : (wpc ? wpc : kMaxWarps[k % kClasses]), c->smem_optin / wbytes)));
+    if (k >= kOwn) continue;
+    share_k[k] = (n_k + most_k[k] - 1) / most_k[k];
+    least += share_k[k];
+  }
+  // (a group of 4 gets an SM for itself where the others leave it one)
+  const int own_sms = std::max(1, sms - n8 - (least + n8 + n4 <= sms ? n4 : (n4 + 1) / 2));
+  if (least <= own_sms) {
+    for (int spare = own_sms - least; spare > 0; --spare) {
+      int best = -1;
+      double last = -1;
+      for (int k = 0; k < kOwn; ++k) {
+        const int n_k = P.first[k + 1] - P.first[k];
+        if (share_k[k] == 0 || share_k[k] >= n_k) continue;
+        // each further string on an SM slows the others by some 8 %: 1000
+        // mixed strings 6.97 us a step (with 15 % 7.29, 25 % 8.0), 256 alike
+        const double est = top[k] * (0.92 + 0.08 * n_k / share_k[k]);
+        if (est > last) last = est, best = k;
+      }
+      if (best < 0) break;
+      ++share_k[best];
+    }
+  } else {
+    for (int k = 0; k < kOwn; ++k)
+      share_k[k] = std::max(1, static_cast<int>(own_sms * (w[k] / std::max(w_all, 1e-300))));
   }
   for (int k = 0; k < kSlots; ++k) {
-    const int n_k = P.first[k + 1] - P.first[k], cls = k % kClasses;
-    P.group[k] = k >= kClasses ? 4 : 1;
+    const int n_k = P.first[k + 1] - P.first[k], most = most_k[k];
+    P.group[k] = k / kClasses == kGroup8 ? 8 : k / kClasses == kGroup4 ? 4 : 1;
     if (n_k == 0) continue;
     Job* const J = &P.jobs[P.first[k]];
-    const size_t wbytes = static_cast<size_t>(P.wf[k]) * sizeof(float);
-    const int most = static_cast<int>(std::max<size_t>(1, std::min<size_t>(
-        k >= kClasses ? 1 : (wpc ? wpc : kMaxWarps[cls]), c->smem_optin / wbytes)));
     int longest = 1;
-    P.ctas[k] = 0;
-    if (k >= kClasses || wpc) {   // groups, or as asked
+    if (k >= kOwn || wpc) {   // groups, or as asked
       longest = most;
       for (int j = 0; j < n_k; j += most) J[P.ctas[k]++].seg = j;
     } else {
-      int share = n_own <= own_sms ? n_k : static_cast<int>(own_sms * (w[k] / std::max(w_all, 1e-300)));
-      share = std::max(1, std::min(share, n_k));
+      const int share = std::min(share_k[k], n_k);
       // segments of equal cost, of no more strings than the fewest rounds hold
-      const int per_cta = (n_k + share - 1) / share, rounds = (per_cta + most - 1) / most;
+      const int per_cta = (n_k + share - 1) / share, rounds = (per_cta + most - 1) / most, cap = rounds * most;
       double left = 0;
       for (int j = 0; j < n_k; ++j) left += cost[order[P.first[k] + j]];
       for (int j = 0; j < n_k;) {
-        const double part = left / std::max(1, std::min(share - P.ctas[k], n_k - j));
-        const int begin = j;
+        const int others = std::max(0, std::min(share - P.ctas[k], n_k - j) - 1);   // segments after this one
+        const double part = left / (others + 1);
+        const int begin = j, must = n_k - j - others * cap;   // (what they cannot hold)
         double sum = 0;
-        while (j < n_k && j - begin < rounds * most) {
+        while (j < n_k && j - begin < cap) {
           const double cj = cost[order[P.first[k] + j]];
-          if (j > begin && sum + 0.5 * cj > part) break;
+          if (j > begin && j - begin >= must && sum + 0.5 * cj > part) break;
           sum += cj;
           ++j;
         }
@@ -900,7 +960,13 @@ sfd_status make_plan(const sfd_ctx* c, const std::vector<Job>& jobs, const std::
     P.regions[k] = std::min(most, longest);
     P.queued[k] = longest > P.regions[k];
   }
-  return SFD_OK;
+  // When there is an SM for every CTA, each asks for more than half of an
+  // SM's shared memory: kernels launched side by side otherwise put CTAs on
+  // the same SM while others idle.
+  int n_ctas = 0;
+  for (int k = 0; k < kSlots; ++k) n_ctas += P.ctas[k];
+  P.smem_least = !wpc && n_ctas <= sms ? static_cast<int>(c->smem_optin / 2) + 1024 : 0;
+  return ensure_slots(c, P);
 }
 
 // Issue the plan's kernels on the context stream (job table already in
@@ -925,7 +991,7 @@ sfd_status issue_plan(sfd_ctx* c, const Plan& P, const Job* d_jobs) {
     }
     if (c->timing) SFD_CUDA(cudaEventRecord(c->t0[k], st));
     cudaError_t e = kLaunch[k % kClasses](d_jobs + P.first[k], n_k, c->d_counter + k * c->sm_count, P.wf[k],
-                               P.regions[k] * P.group[k], P.ctas[k], P.queued[k], P.group[k], st);
+                               P.regions[k] * P.group[k], P.ctas[k], P.queued[k], P.group[k], P.smem_least, st);
     if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
     if (c->timing) {
       SFD_CUDA(cudaEventRecord(c->t1[k], st));
@@ -1155,11 +1221,6 @@ sfd_status sfd_ctx_create(int device, void* cuda_stream, size_t mem_budget_bytes
   bool ok = cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) == cudaSuccess &&
             cudaEventCreateWithFlags(&c->copied, cudaEventDisableTiming) == cudaSuccess &&
             cudaStreamCreateWithFlags(&c->copy, cudaStreamNonBlocking) == cudaSuccess;
-  for (int k = 0; k < kSlots && ok; ++k) {
-    ok = cudaStreamCreateWithFlags(&c->side[k], cudaStreamNonBlocking) == cudaSuccess &&
-         cudaEventCreateWithFlags(&c->join[k], cudaEventDisableTiming) == cudaSuccess &&
-         cudaEventCreate(&c->t0[k]) == cudaSuccess && cudaEventCreate(&c->t1[k]) == cudaSuccess;
-  }
   if (!ok) {
     sfd_ctx_destroy(c);
     return fail(SFD_ECUDA, "stream/event creation failed");
@@ -1925,7 +1986,7 @@ sfd_status sfd_batch_autotune(sfd_batch* b, int64_t probe_samples, int32_t* best
   cudaEventCreate(&e1);
   float best_ms = 0.f;
   int best = 0, best_groups = 0;
-  const int candidates[4] = {1, 2, 4, 0};   // 0: automatic (reported as 4)
+  const int candidates[3] = {1, 2, 4};
   // warp groups are a candidate only if they would form for this batch
   bool groups_form = false;
   {
@@ -1933,11 +1994,10 @@ sfd_status sfd_batch_autotune(sfd_batch* b, int64_t probe_samples, int32_t* best
     std::vector<const sfd_string*> owners(b->strings.begin(), b->strings.end());
     Plan P;
     if (make_plan(c, jobs, owners, 0, P, 1) == SFD_OK)
-      groups_form = P.first[kSlots] > P.first[kClasses];
+      groups_form = P.first[kSlots] > P.first[kGroup4 * kClasses];
   }
-  int best_wpc = 0;
-  for (int cj = 0; cj < 8 && rc == SFD_OK; ++cj) {
-    const int ci = cj % 4, groups = cj / 4;   // warps per CTA x warp groups off / on
+  for (int cj = 0; cj < 6 && rc == SFD_OK; ++cj) {
+    const int ci = cj % 3, groups = cj / 3;   // warps per CTA x warp groups off / on
     if (groups && !groups_form) continue;
     // fresh clones of the current state for every candidate
     std::vector<sfd_string*> cl;
@@ -1964,12 +2024,7 @@ sfd_status sfd_batch_autotune(sfd_batch* b, int64_t probe_samples, int32_t* best
         float ms = 0.f;
         if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
         if (e != cudaSuccess) rc = cuda_fail(e, "autotune timing");
-        else if (best == 0 || ms < best_ms) {
-          best_ms = ms;
-          best_wpc = candidates[ci];
-          best = best_wpc ? best_wpc : 4;
-          best_groups = groups;
-        }
+        else if (best == 0 || ms < best_ms) { best_ms = ms; best = candidates[ci]; best_groups = groups; }
       }
     }
     cudaStreamSynchronize(c->stream);
@@ -1979,7 +2034,7 @@ sfd_status sfd_batch_autotune(sfd_batch* b, int64_t probe_samples, int32_t* best
   cudaEventDestroy(e1);
   c->pool.dealloc(dout);
   if (rc) return rc;
-  b->wpc = best_wpc;
+  b->wpc = best;
   b->groups = best_groups;
   if (best_warps_per_cta) *best_warps_per_cta = best;
   return SFD_OK;
@@ -2139,7 +2194,7 @@ extern "C" sfd_status sfd_synthesize_noalloc(int device, void* cuda_stream, cons
   const int k = job_class(D);
   int* counter = reinterpret_cast<int*>(b + o_cnt) + k;   // the launcher clears it on `stream`
   e = kLaunch[k](reinterpret_cast<const Job*>(b + o_job), 1, counter,
-                 warp_smem_floats(D.m_u, D.m_z, D.z_jacobi), 1, 1, 0, 1, stream);
+                 warp_smem_floats(D.m_u, D.m_z, D.z_jacobi), 1, 1, 0, 1, 0, stream);
   if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
   e = cudaMemcpyAsync(&sc, b + o_sc, sizeof(Scalars), cudaMemcpyDeviceToHost, stream);
   if (e != cudaSuccess) return cuda_fail(e, "status read");

@@ -26,6 +26,7 @@
 // through the unit-force response A^{-1} J solved alongside.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "sfd_step_smem.cuh"
@@ -67,26 +68,23 @@ constexpr int kMaxThreads = kWarp * 4;
 // step strings of one or two kinds: each instance's time loop is 10-25 KB of
 // code, and with the kinds mixed on every SM (one queue for all CTAs) their
 // instruction fetches missed the cache: 1000 mixed strings then took 14.3 us
-// a step, in segments 8.8 us (one generic loop for every kind: 10.0 us).
+// a step, in segments 8.8 us (7.0 us with every later change; one generic
+// loop for every kind: 10.0 us).
 //
-// With group = 2 or 4 (register path only, at most 4 warps per CTA; the
-// host launches groups of 4) the
-// CTA's warps work in groups (warps g*group .. g*group + group - 1 share
-// region g): the group's first warp takes the next job and passes it on
-// through shared memory (named barrier 1 + g over the whole group), and the
-// warps the job can use step it (run_job_reg, in-job barrier 1 + g for
-// pairs, 3 for groups of 4, whose unused warps meanwhile wait at barrier 1).
-// The job index cells alternate so that a cell is rewritten only after every
-// warp of the group has passed the next barrier, i.e. after all have read it.
+// With group = 4 or 8 (register path only) the CTA's warps step one string at
+// a time together: warp 0 takes the next job and passes it on through shared
+// memory (jcell) behind the group's barrier.  The cells alternate so that one
+// is rewritten only after every warp has passed the next barrier, i.e. after
+// all have read it.
 __global__ void __launch_bounds__(kMaxThreads, 1) SFD_KERNEL(const Job* __restrict__ jobs, int n_jobs,
                                                              int* __restrict__ counters, int warp_floats,
                                                              int queued, int group) {
   extern __shared__ float smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & (kWarp - 1);
 #ifdef SFD_MU
-  __shared__ __align__(16) float xcells[2][1024];  // per group: [buffer][warp][chg, mag, chx, mgx][lane]
-  __shared__ int jcell[2][2];        // per group: job index, alternating
-  const int npw = group == 4 ? 4 : (group == 2 ? 2 : 1);
+  __shared__ __align__(16) float xcells[2048];   // [buffer][warp][lane][chg, mag, chx, mgx]
+  __shared__ int jcell[2];                       // a group's job index, alternating
+  const int npw = group;
 #else
   const int npw = 1;
   (void)group;
@@ -132,15 +130,15 @@ __global__ void __launch_bounds__(kMaxThreads, 1) SFD_KERNEL(const Job* __restri
     if (pw == 0) j = next_job(first);
 #ifdef SFD_MU
     if (npw > 1) {
-      if (pw == 0 && lane == 0) jcell[pi][it & 1] = j;
-      group_sync(1 + pi, npw);
-      j = jcell[pi][it & 1];
+      if (pw == 0 && lane == 0) jcell[it & 1] = j;
+      group_sync(npw);
+      j = jcell[it & 1];
       ++it;
     }
 #endif
     if (j >= n_jobs) break;
 #ifdef SFD_MU
-    run_job_reg<SFD_MU>(jobs[j], region, lane, pw, npw, npw == 4 ? 3 : 1 + pi, npw > 1 ? xcells[pi] : nullptr);
+    run_job_reg<SFD_MU>(jobs[j], region, lane, pw, npw, xcells);
 #else
     run_job(jobs[j], smem + region, lane);
 #endif
@@ -182,20 +180,19 @@ cudaError_t raise_smem_limit() {
 // c steps its segment of the jobs, warps_per_cta / group of them at a time.
 // With `queued` (some segment is longer than that) the CTAs take them by one
 // counter each, cleared on the same stream before the kernel starts.  With
-// group = 2 or 4 (register classes; at most 4 warps per CTA, a multiple of
-// it) each string gets a group of warps and one shared-memory region per
-// group.
+// group = 4 or 8 (register classes; warps_per_cta = group) each string gets
+// the CTA's warps and one shared-memory region.
 cudaError_t SFD_LAUNCHER(const Job* d_jobs, int n_jobs, int* d_counters, int warp_floats, int warps_per_cta,
-                         int n_ctas, int queued, int group, cudaStream_t stream) {
+                         int n_ctas, int queued, int group, int smem_least, cudaStream_t stream) {
 #ifndef SFD_MU
   group = 1;
 #endif
-  if (group != 1 && group != 2 && group != 4) return cudaErrorInvalidValue;
-  if (warps_per_cta < 1 || warps_per_cta * kWarp > kMaxThreads || warps_per_cta % group != 0 ||
-      (group > 1 && warps_per_cta > 4))
+  if (group != 1 && group != 4 && group != 8) return cudaErrorInvalidValue;
+  if (warps_per_cta < 1 || warps_per_cta * kWarp > kMaxThreads || (group > 1 && warps_per_cta != group))
     return cudaErrorInvalidValue;
   const int regions = warps_per_cta / group;
-  const size_t smem = static_cast<size_t>(warp_floats) * regions * sizeof(float);
+  const size_t smem = std::max(static_cast<size_t>(warp_floats) * regions * sizeof(float),
+                               static_cast<size_t>(smem_least));
   cudaError_t e = raise_smem_limit();
   if (e != cudaSuccess) return e;
   if (queued) {

@@ -268,46 +268,39 @@ __device__ __forceinline__ void tri_solve_r(const float (&sb)[MU], const float (
   }
 }
 
-// Barrier of the ng warps stepping one string together (named barrier id
-// 1-3, 32 ng threads).  Ids and counts are immediates, so the kernel
-// reserves only those barriers.
-__device__ __forceinline__ void group_sync(int id, int ng) {
-  if (ng == 4) {
-    if (id == 3) asm volatile("bar.sync 3, 128;" ::: "memory");
-    else asm volatile("bar.sync 1, 128;" ::: "memory");
-  } else {
-    if (id == 1) asm volatile("bar.sync 1, 64;" ::: "memory");
-    else if (id == 2) asm volatile("bar.sync 2, 64;" ::: "memory");
-    else asm volatile("bar.sync 3, 64;" ::: "memory");
-  }
+// Barrier of the ng = 4 or 8 warps stepping one string together (named
+// barrier 1).  Id and counts are immediates, so the kernel reserves only that
+// barrier.
+__device__ __forceinline__ void group_sync(int ng) {
+  if (ng == 8) asm volatile("bar.sync 1, 256;" ::: "memory");
+  else asm volatile("bar.sync 1, 128;" ::: "memory");
 }
 
-// A string may be stepped by one warp or by a group of ng = 2 or 4 warps of
-// one CTA (warp pw of the group; the group launched with npw warps shares
-// the string's shared-memory region, named barrier bar_id and exchange
-// cells xcell[1024]).  Every warp of a group does the whole transverse side
-// identically (same data, same operations, so the same bits), and the
-// group splits the longitudinal rows by k mod ng; the warps meet at a
-// barrier once the state is loaded, once the longitudinal right-hand side
-// is formed (its transfer slots are written again in the sweeps), once per
-// Gauss-Seidel sweep (where they also take the maximum of each lane's
-// convergence measures, so all see exactly what one warp over all rows
-// would) and once per step after the longitudinal update.  Every barrier
-// sits in control flow that depends only on that shared data.  Only strings
-// whose longitudinal grid is folded into the sweeps (z_jacobi) with at least
-// 5 rows per lane take a group; the launch's other warps return at once.
+// A string may be stepped by one warp or by a group of ng = 4 or 8 warps, all
+// of one CTA (this one is warp pw; they share the string's shared-memory
+// region and the exchange cells xcell, 256 floats per warp).  Every warp of a
+// group does the whole transverse side identically (same data, same
+// operations, so the same bits), and the group splits the longitudinal rows
+// by k mod ng; the warps meet at a barrier once the state is loaded, once the
+// longitudinal right-hand side is formed (its transfer slots are written
+// again in the sweeps), once per Gauss-Seidel sweep (where they also take the
+// maximum of each lane's convergence measures, so all see exactly what one
+// warp over all rows would) and once per step after the longitudinal update.
+// Every barrier sits in control flow that depends only on that shared data.
+// Only strings whose longitudinal grid is folded into the sweeps (z_jacobi)
+// and gives every warp a row take a group; in a CTA launched for groups
+// another string is stepped by warp 0 while the others return at once.
 // Warp 0 of a group writes the output, the trajectory record and the state.
 constexpr uint32_t kSweepFlush = 1u << 30;
 
 struct WarpGroup {
   int pw = 0, ng = 1;            // this warp's place in the group stepping the string
-  int bar_id = 1;
   float* xcell = nullptr;
 };
 
 // One job of one string.  MZ: longitudinal rows per lane held in registers
-// (0: no longitudinal grid; 1 or 3, folded into the sweeps, one warp; 403: up
-// to 12, three in the registers of each of a group's 4 warps), -1 for
+// (0: no longitudinal grid; 1 or 3, folded into the sweeps, one warp; 403, 803:
+// up to 12 or 24, three in the registers of each of a group's 4 or 8 warps), -1 for
 // any number kept in shared memory (folded, warp groups), -2 for a factored
 // longitudinal matrix (shared memory, one warp).
 // Not inlined: each instance gets its own registers (inlined side by side in
@@ -370,7 +363,7 @@ __device__ __noinline__ void step_string(const Job& job, int region, int lane, c
     const int total = static_cast<int>(p - wbase);
     for (int k = 2 * RU + lane + kWarp * kz0; k < total; k += kWarp * kzs) wbase[k] = 0.f;
     __syncwarp();
-    if (paired) group_sync(g.bar_id, g.ng);   // the region is zero before either warp writes to it
+    if (paired) group_sync(g.ng);   // the region is zero before either warp writes to it
   }
   // value of a field at longitudinal row i
   auto zat = [&](int field, const float* A, int i) {
@@ -470,7 +463,7 @@ __device__ __noinline__ void step_string(const Job& job, int region, int lane, c
   // string's total every kSweepFlush steps and at the end)
   uint32_t sweeps_sum = 0;
   __syncwarp();
-  if (paired) group_sync(g.bar_id, g.ng);   // both halves of the longitudinal state are loaded
+  if (paired) group_sync(g.ng);   // both halves of the longitudinal state are loaded
 
   // (P^T F) at longitudinal node m = sum over the transverse nodes l of
   // P[l, m] F_l, P the linear interpolation from the longitudinal to the
@@ -878,7 +871,7 @@ __device__ __noinline__ void step_string(const Job& job, int region, int lane, c
           for (int q = 0; q < R; ++q) sts<oRZ>(a[q], v[q]);
         });
         __syncwarp();
-        if (paired) group_sync(g.bar_id, g.ng);   // every warp has read the slots that the sweeps rewrite
+        if (paired) group_sync(g.ng);   // every warp has read the slots that the sweeps rewrite
       } else {
         static_for<NZ>([&](auto kc) {
           constexpr int k = decltype(kc)::value;
@@ -888,7 +881,7 @@ __device__ __noinline__ void step_string(const Job& job, int region, int lane, c
         });
         if (paired) {
           __syncwarp();
-          group_sync(g.bar_id, g.ng);
+          group_sync(g.ng);
         }
       }
       // ---- stage 3: block Gauss-Seidel on (a, az) [and the response] ----
@@ -1050,11 +1043,11 @@ __device__ __noinline__ void step_string(const Job& job, int region, int lane, c
           if (paired) {
             // each lane's maxima over the group's rows: the other warps'
             // updates are in shared memory once all pass the barrier
-            float4* xc = reinterpret_cast<float4*>(g.xcell) + xpar * 128 + lane;
+            float4* xc = reinterpret_cast<float4*>(g.xcell) + xpar * (kNG > 1 ? 32 * kNG : 32 * g.ng) + lane;
             xc[g.pw * 32] = make_float4(chg, mag, chx, mgx);
-            group_sync(g.bar_id, g.ng);
+            group_sync(g.ng);
 #pragma unroll
-            for (int w = 0; w < 4; ++w) {
+            for (int w = 0; w < 8; ++w) {
               if (w >= (kNG > 1 ? kNG : g.ng)) break;
               const float4 o = xc[w * 32];
               chg = fmaxf(chg, o.x);
@@ -1176,7 +1169,7 @@ __device__ __noinline__ void step_string(const Job& job, int region, int lane, c
     }
     const bool unstable = __any_sync(SFD_FULL, bad);
     if (kHasZ) __syncwarp();
-    if (paired) group_sync(g.bar_id, g.ng);   // the new level is complete in shared memory
+    if (paired) group_sync(g.ng);   // the new level is complete in shared memory
     ++n;
     if (recorded && writer) {   // record for the adjoint: the new level
       const Job* J = reread(&job);
@@ -1251,7 +1244,7 @@ __device__ __forceinline__ void run_job_exc(const Job& job, int region, int lane
   const Desc* __restrict__ Dp = job.desc;
   const int m_z = Dp->m_z;
   const bool zjac = Dp->z_jacobi != 0;
-  if (npw >= 2 && zjac && m_z >= 5) g.ng = npw;
+  if (npw > 1 && zjac && m_z >= npw) g.ng = npw;   // (a row for every warp)
   if (g.pw >= g.ng) return;                       // the group's other warps step it
   if (Dp->linear) step_string<MU, 0, EXC, true>(job, region, lane, g);
   else if (m_z == 0) step_string<MU, 0, EXC, false>(job, region, lane, g);
@@ -1259,15 +1252,14 @@ __device__ __forceinline__ void run_job_exc(const Job& job, int region, int lane
   else if (m_z == 1) step_string<MU, 1, EXC, false>(job, region, lane, g);
   else if (m_z == 3) step_string<MU, 3, EXC, false>(job, region, lane, g);
   else if (g.ng == 4 && m_z <= 12) step_string<MU, 403, EXC, false>(job, region, lane, g);
+  else if (g.ng == 8 && m_z > 8 && m_z <= 24) step_string<MU, 803, EXC, false>(job, region, lane, g);
   else step_string<MU, -1, EXC, false>(job, region, lane, g);
 }
 
 template <int MU>
-__device__ __forceinline__ void run_job_reg(const Job& job, int region, int lane, int pw, int npw, int bar_id,
-                                            float* xcell) {
+__device__ __forceinline__ void run_job_reg(const Job& job, int region, int lane, int pw, int npw, float* xcell) {
   WarpGroup g;
   g.pw = pw;
-  g.bar_id = bar_id;
   g.xcell = xcell;
   const int exc = job.desc->exc;
   if (exc == kPluck) run_job_exc<MU, kPluck>(job, region, lane, g, npw);
