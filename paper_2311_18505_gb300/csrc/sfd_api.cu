@@ -962,7 +962,8 @@ sfd_status make_plan(sfd_ctx* c, const std::vector<Job>& jobs, const std::vector
   }
   // When there is an SM for every CTA, each asks for more than half of an
   // SM's shared memory: kernels launched side by side otherwise put CTAs on
-  // the same SM while others idle.
+  // the same SM while others idle (256 mixed strings 4.87 ms a block of 1024
+  // without, 4.36 with).
   int n_ctas = 0;
   for (int k = 0; k < kSlots; ++k) n_ctas += P.ctas[k];
   P.smem_least = !wpc && n_ctas <= sms ? static_cast<int>(c->smem_optin / 2) + 1024 : 0;
