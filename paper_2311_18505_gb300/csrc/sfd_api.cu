@@ -880,14 +880,12 @@ sfd_status make_plan(sfd_ctx* c, const std::vector<Job>& jobs, const std::vector
   const int n4 = P.first[kGroup8 * kClasses] - P.first[kGroup4 * kClasses];
   const int n8 = P.first[kSlots] - P.first[kGroup8 * kClasses];
   constexpr int kOwn = kGroup4 * kClasses;   // slots below: a warp per string
-  double w_all = 0, w[kSlots] = {};   // SM time: a string holds 1 / kMaxWarps of one
+  // SM time: a string holds 1 / most_k of one, most_k being what registers and
+  // shared memory let an SM step at once (by registers alone the strings of
+  // many longitudinal rows got too few SMs and the 4096-string batch waited
+  // for them: 3.52 s a batch of 4 s, 3.10 s so)
+  double w_all = 0, w[kSlots] = {};
   double top[kSlots] = {};            // the slot's longest job
-  for (int i = 0; i < nj; ++i) {
-    const int k = slot[i];
-    w[k] += cost[i] / kMaxWarps[k % kClasses];
-    top[k] = std::max(top[k], cost[i]);
-    if (k < kOwn) w_all += cost[i] / kMaxWarps[k % kClasses];
-  }
   // SMs per slot: when one round holds every string, at least what that
   // takes, the others to whichever slot would end last; else by cost
   int most_k[kSlots] = {}, share_k[kSlots] = {}, least = 0;
@@ -900,6 +898,11 @@ sfd_status make_plan(sfd_ctx* c, const std::vector<Job>& jobs, const std::vector
     if (k >= kOwn) continue;
     share_k[k] = (n_k + most_k[k] - 1) / most_k[k];
     least += share_k[k];
+  }
+  for (int i = 0; i < nj; ++i) {
+    const int k = slot[i];
+    top[k] = std::max(top[k], cost[i]);
+    if (k < kOwn) w[k] += cost[i] / most_k[k], w_all += cost[i] / most_k[k];
   }
   // (a group of 4 gets an SM for itself where the others leave it one)
   const int own_sms = std::max(1, sms - n8 - (least + n8 + n4 <= sms ? n4 : (n4 + 1) / 2));
