@@ -739,8 +739,9 @@ __device__ __noinline__ void step_string(const Job& job, int region, int lane, c
   // gamma^2 coefficients of the step (constant without f0 modulation)
   float lam2 = Dp->lam2, lam2_lo = Dp->lam2_lo, lam2l = Dp->lam2l, ca = Dp->ca, cb = Dp->cb, cz = Dp->cz;
 
-  // jnext = n + 1 from here: each step reaches the level of one sample
-  const int64_t n_end = j_end - 1;
+  // jnext = n + 1 from here: each step reaches the level of one sample.  (A
+  // string already unstable has had its zeros and is not stepped again.)
+  const int64_t n_end = (status & kStUnstable) ? n : j_end - 1;
   while (n < n_end) {
     // ======================= one step n -> n+1 =======================
     if (mod_kind != 0) {
