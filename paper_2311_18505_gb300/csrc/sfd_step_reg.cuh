@@ -302,8 +302,8 @@ struct WarpGroup {
   float* xcell = nullptr;
 };
 
-// One job of one string.  MZ: longitudinal rows per lane held in registers
-// (0: no longitudinal grid; 1 or 3, folded into the sweeps, one warp; 403, 803:
+// One job of one string that is not unstable yet.  MZ: longitudinal rows per
+// lane held in registers (0: no longitudinal grid; 1 or 3, folded into the sweeps, one warp; 403, 803:
 // up to 12 or 24, three in the registers of each of a group's 4 or 8 warps), -1 for
 // any number kept in shared memory (folded, warp groups), -2 for a factored
 // longitudinal matrix (shared memory, one warp).
@@ -730,18 +730,17 @@ __device__ __noinline__ void step_string(const Job& job, int region, int lane, c
     }
   };
 
-  // the levels already reached (at most two samples), or zeros once unstable
-  while (jnext < j_end && (jnext <= n || (status & kStUnstable))) {
-    put((status & kStUnstable) ? 0.f : sample(jnext == n - 1));
+  // the levels already reached (at most two samples)
+  while (jnext < j_end && jnext <= n) {
+    put(sample(jnext == n - 1));
     ++jnext;
   }
 
   // gamma^2 coefficients of the step (constant without f0 modulation)
   float lam2 = Dp->lam2, lam2_lo = Dp->lam2_lo, lam2l = Dp->lam2l, ca = Dp->ca, cb = Dp->cb, cz = Dp->cz;
 
-  // jnext = n + 1 from here: each step reaches the level of one sample.  (A
-  // string already unstable has had its zeros and is not stepped again.)
-  const int64_t n_end = (status & kStUnstable) ? n : j_end - 1;
+  // jnext = n + 1 from here: each step reaches the level of one sample
+  const int64_t n_end = j_end - 1;
   while (n < n_end) {
     // ======================= one step n -> n+1 =======================
     if (mod_kind != 0) {
