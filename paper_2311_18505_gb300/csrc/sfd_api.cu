@@ -23,7 +23,7 @@
 namespace sfd {
 #define SFD_DECLARE_LAUNCHER(name)                                                                   \
   cudaError_t name(const Job* d_jobs, int n_jobs, int* d_counter, int warp_floats, int warps_per_cta, \
-                   int n_ctas, int queued, int group, int smem_least, cudaStream_t stream);
+                   int n_ctas, int queued, int group, int priority, cudaStream_t stream);
 SFD_DECLARE_LAUNCHER(launch_synth_reg1)
 SFD_DECLARE_LAUNCHER(launch_synth_reg3)
 SFD_DECLARE_LAUNCHER(launch_synth_reg5)
@@ -145,6 +145,7 @@ struct sfd_ctx {
   int timed_jobs[kSlots] = {};           // jobs of each slot in the last launch
   Pool pool;
   int sm_count = 0;
+  int priority = 0;                        // of small launches (small_priority)
   size_t smem_optin = 0;
   int warp_pairs = 1;                      // 0: every string on one warp (sfd_ctx_set_warp_pairs)
   int sweep_cap = 0;                       // coupled-solve sweep cap of every launch (0: kMaxSweeps)
@@ -757,6 +758,8 @@ const int kMaxWarps[kClasses] = {16, 8, 8, 8, 8, 4};
 // registers of each: 5.3-5.5 us a step, in groups of 4 6.1-6.3 (bowed, 17 and
 // 19 rows; from 29 rows on, more warps gain nothing)
 constexpr int kWideRows = 13, kWideMost = 24;
+// SMs that a batch of fewer CTAs than SMs leaves to others (make_plan)
+constexpr int kFreeSms = 2;
 const Launcher kLaunch[kClasses] = {launch_synth_reg1, launch_synth_reg3, launch_synth_reg5,
                                     launch_synth_reg7, launch_synth_reg9, launch_synth_smem};
 
@@ -767,12 +770,12 @@ struct Plan {
   std::vector<Job> jobs;
   int first[kSlots + 1] = {};
   int wf[kSlots] = {};
-  int group[kSlots] = {};       // warps per string of the slot's launch (1, 2 or 4)
+  int group[kSlots] = {};       // warps per string of the slot's launch (1, 4 or 8)
   int regions[kSlots] = {};     // strings stepped at a time by a CTA
   int queued[kSlots] = {};      // some segment is longer than that
   int ctas[kSlots] = {};
-  int order[kSlots] = {};       // launch order of the slots: heaviest step first
-  int smem_least = 0;           // shared memory a CTA asks for at least (no two on an SM)
+  int order[kSlots] = {};       // launch order of the slots
+  bool small = false;           // a launch of few CTAs: placed before a larger one's waiting CTAs
 };
 
 // The side stream and events of every slot the plan uses, made on the slot's
@@ -861,8 +864,9 @@ sfd_status make_plan(sfd_ctx* c, const std::vector<Job>& jobs, const std::vector
     if (static_cast<size_t>(P.wf[k]) * sizeof(float) > c->smem_optin)
       return fail(SFD_EINVAL, "string too large for one warp's shared memory");
   }
-  // Slots are launched heaviest step first (groups, then many longitudinal
-  // rows, then shared-memory grids and 9, 7, 5, 3, 1 transverse rows per lane).  The block scheduler starts CTAs in
+  // A batch of more CTAs than SMs is launched heaviest step first (groups,
+  // then many longitudinal rows, then shared-memory grids and 9, 7, 5, 3, 1
+  // transverse rows per lane).  The block scheduler starts CTAs in
   // launch order, and a class's CTAs keep taking its jobs until none is left,
   // so when the batch does not fit on the GPU at once the class launched
   // first holds the SMs; launched last, the slowest strings would start only
@@ -907,7 +911,13 @@ sfd_status make_plan(sfd_ctx* c, const std::vector<Job>& jobs, const std::vector
   // (a group of 4 gets an SM for itself where the others leave it one)
   const int own_sms = std::max(1, sms - n8 - (least + n8 + n4 <= sms ? n4 : (n4 + 1) / 2));
   if (least <= own_sms) {
-    for (int spare = own_sms - least; spare > 0; --spare) {
+    // Where an SM is left for every CTA, kFreeSms get none: a CTA of another
+    // context that needs a whole SM (a group of 8) then starts at once.  64
+    // strings of 40-1000 Hz x 256 samples beside a batch of 256 x 8192 take
+    // 1.6 ms so, 11.8 without.  The batch itself: 5.19 ms a block of 1024 with
+    // no SM left free, 5.31 with 2, 5.37 with 4 (mean of ten sets of strings).
+    const int keep = least + n4 + n8 + kFreeSms <= sms ? kFreeSms : 0;
+    for (int spare = own_sms - least - keep; spare > 0; --spare) {
       int best = -1;
       double last = -1;
       for (int k = 0; k < kOwn; ++k) {
@@ -963,14 +973,36 @@ sfd_status make_plan(sfd_ctx* c, const std::vector<Job>& jobs, const std::vector
     P.regions[k] = std::min(most, longest);
     P.queued[k] = longest > P.regions[k];
   }
-  // When there is an SM for every CTA, each asks for more than half of an
-  // SM's shared memory: kernels launched side by side otherwise put CTAs on
-  // the same SM while others idle (256 mixed strings 4.87 ms a block of 1024
-  // without, 4.36 with).
   int n_ctas = 0;
   for (int k = 0; k < kSlots; ++k) n_ctas += P.ctas[k];
-  P.smem_least = !wpc && n_ctas <= sms ? static_cast<int>(c->smem_optin / 2) + 1024 : 0;
+  // A batch with an SM for every CTA is launched largest CTA first (by the
+  // registers of its warps): in any other order the block scheduler puts CTAs
+  // of one launch beside a smaller one of another while SMs idle (256 mixed
+  // strings 4.93 ms a block of 1024 heaviest step first, 4.38 so).  CTAs that
+  // each ask for half an SM's shared memory stay apart as well and gain the
+  // same, but then no other context's CTA fits beside them: a one-note call
+  // beside a batch of 256 x 8192 samples took 11.0 ms, takes 0.24 (alone 0.21).
+  if (n_ctas <= sms && !wpc) {
+    auto share = [&](int k) { return P.regions[k] * P.group[k] * (kMaxWarps[0] / kMaxWarps[k % kClasses]); };
+    std::stable_sort(P.order, P.order + kSlots, [&](int x, int y) { return share(x) > share(y); });
+  }
+  P.small = n_ctas <= sms / 2;
   return ensure_slots(c, P);
+}
+
+// Launch priority of small plans on `stream` (0: none): one above a stream's
+// default, or the stream's own where that is higher.  CTAs of a batch that
+// wait for a free SM hold up every launch behind them, also one whose CTAs
+// would fit beside those already running: a one-note call beside a batch of
+// 1000 strings x 8192 samples took 17.4 ms, with priority 0.41, six notes 17.6
+// and 0.46.  (Launching such a batch largest CTA first leaves none waiting and
+// the note 0.28 ms, but costs the batch 8 %: 3.90 to 4.22 ms for 512 samples.)
+int small_priority(cudaStream_t stream) {
+  int least = 0, greatest = 0, own = 0;
+  const bool ok = cudaDeviceGetStreamPriorityRange(&least, &greatest) == cudaSuccess &&
+                  cudaStreamGetPriority(stream, &own) == cudaSuccess;
+  if (!ok) cudaGetLastError();
+  return ok ? std::min(own, std::max(greatest, least - 1)) : 0;
 }
 
 // Issue the plan's kernels on the context stream (job table already in
@@ -995,7 +1027,8 @@ sfd_status issue_plan(sfd_ctx* c, const Plan& P, const Job* d_jobs) {
     }
     if (c->timing) SFD_CUDA(cudaEventRecord(c->t0[k], st));
     cudaError_t e = kLaunch[k % kClasses](d_jobs + P.first[k], n_k, c->d_counter + k * c->sm_count, P.wf[k],
-                               P.regions[k] * P.group[k], P.ctas[k], P.queued[k], P.group[k], P.smem_least, st);
+                               P.regions[k] * P.group[k], P.ctas[k], P.queued[k], P.group[k], P.small ? c->priority : 0,
+                               st);
     if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
     if (c->timing) {
       SFD_CUDA(cudaEventRecord(c->t1[k], st));
@@ -1215,6 +1248,7 @@ sfd_status sfd_ctx_create(int device, void* cuda_stream, size_t mem_budget_bytes
   }
   c->sm_count = prop.multiProcessorCount;
   c->smem_optin = prop.sharedMemPerBlockOptin - kStaticSmemBytes;
+  c->priority = small_priority(c->stream);
   sfd_status rc = c->pool.init(mem_budget_bytes ? mem_budget_bytes : (size_t{256} << 20));
   if (rc) { delete c; return rc; }
   if ((e = cudaMalloc(&c->d_counter, sizeof(int) * kSlots * c->sm_count)) != cudaSuccess) {
@@ -2198,7 +2232,7 @@ extern "C" sfd_status sfd_synthesize_noalloc(int device, void* cuda_stream, cons
   const int k = job_class(D);
   int* counter = reinterpret_cast<int*>(b + o_cnt) + k;   // the launcher clears it on `stream`
   e = kLaunch[k](reinterpret_cast<const Job*>(b + o_job), 1, counter,
-                 warp_smem_floats(D.m_u, D.m_z, D.z_jacobi), 1, 1, 0, 1, 0, stream);
+                 warp_smem_floats(D.m_u, D.m_z, D.z_jacobi), 1, 1, 0, 1, small_priority(stream), stream);
   if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
   e = cudaMemcpyAsync(&sc, b + o_sc, sizeof(Scalars), cudaMemcpyDeviceToHost, stream);
   if (e != cudaSuccess) return cuda_fail(e, "status read");

@@ -26,7 +26,6 @@
 // through the unit-force response A^{-1} J solved alongside.
 #include <cuda_runtime.h>
 
-#include <algorithm>
 #include <mutex>
 
 #include "sfd_step_smem.cuh"
@@ -184,6 +183,16 @@ cudaError_t raise_smem_limit() {
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(SFD_KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            optin - static_cast<int>(fa.sharedSizeBytes));
+  if (e != cudaSuccess) return e;
+  // One division of an SM's L1 for the launches of all classes.  Left to the
+  // runtime it follows each launch's own need, and an SM that runs CTAs under
+  // one division starts none that want another until it is empty: with a
+  // group of 4 warps on every SM, half of its registers free, a one-note call
+  // of another context waited 39 ms for the first to end, now takes 0.3 (alone
+  // 0.2).  164 of 228 KB for shared memory: with all of it the spills of the
+  // widest instances miss what is left (96 kHz bass strings 8.25 -> 8.62 ms a
+  // block of 1024), with 164, 132 or the runtime's choice they take the same.
+  e = cudaFuncSetAttribute(SFD_KERNEL, cudaFuncAttributePreferredSharedMemoryCarveout, 72);
   if (e == cudaSuccess) g_attr_done[dev] = true;
   return e;
 }
@@ -194,9 +203,10 @@ cudaError_t raise_smem_limit() {
 // With `queued` (some segment is longer than that) the CTAs take them by one
 // counter each, cleared on the same stream before the kernel starts.  With
 // group = 4 or 8 (register classes; warps_per_cta = group) each string gets
-// the CTA's warps and one shared-memory region.
+// the CTA's warps and one shared-memory region.  A priority other than 0 is
+// the launch's own, whatever the stream's.
 cudaError_t SFD_LAUNCHER(const Job* d_jobs, int n_jobs, int* d_counters, int warp_floats, int warps_per_cta,
-                         int n_ctas, int queued, int group, int smem_least, cudaStream_t stream) {
+                         int n_ctas, int queued, int group, int priority, cudaStream_t stream) {
 #ifndef SFD_MU
   group = 1;
 #endif
@@ -204,17 +214,26 @@ cudaError_t SFD_LAUNCHER(const Job* d_jobs, int n_jobs, int* d_counters, int war
   if (warps_per_cta < 1 || warps_per_cta * kWarp > kMaxThreads || (group > 1 && warps_per_cta != group))
     return cudaErrorInvalidValue;
   const int regions = warps_per_cta / group;
-  const size_t smem = std::max(static_cast<size_t>(warp_floats) * regions * sizeof(float),
-                               static_cast<size_t>(smem_least));
+  const size_t smem = static_cast<size_t>(warp_floats) * regions * sizeof(float);
   cudaError_t e = raise_smem_limit();
   if (e != cudaSuccess) return e;
   if (queued) {
     e = cudaMemsetAsync(d_counters, 0, sizeof(int) * n_ctas, stream);
     if (e != cudaSuccess) return e;
   }
-  SFD_KERNEL<<<n_ctas, warps_per_cta * kWarp, smem, stream>>>(d_jobs, n_jobs, d_counters, warp_floats, queued,
-                                                              group);
-  return cudaGetLastError();
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributePriority;
+  attr.val.priority = priority;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n_ctas);
+  cfg.blockDim = dim3(warps_per_cta * kWarp);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = priority != 0 ? 1 : 0;
+  e = cudaLaunchKernelEx(&cfg, SFD_KERNEL, d_jobs, n_jobs, d_counters, warp_floats, queued, group);
+  const cudaError_t last = cudaGetLastError();   // (cleared, whatever the launch returned)
+  return e != cudaSuccess ? e : last;
 }
 
 }  // namespace sfd
