@@ -136,13 +136,16 @@ constexpr int kSlots = kSlotKinds * kClasses;
 struct sfd_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
-  cudaStream_t side[kSlots] = {};        // one per slot in use (ensure_slots), forked from `stream`
+  // by a launch's place in the plan's order; kClasses of each made with the
+  // context, more when a plan first needs them (ensure_lanes)
+  cudaStream_t side[kSlots] = {};        // forked from `stream`
   cudaEvent_t fork = nullptr, join[kSlots] = {};
   cudaStream_t copy = nullptr;           // host-output copies of classes already ended
   cudaEvent_t copied = nullptr;          // end of those copies, joined back to `stream`
   bool timing = false;                   // record per-class kernel times
   cudaEvent_t t0[kSlots] = {}, t1[kSlots] = {};
-  int timed_jobs[kSlots] = {};           // jobs of each slot in the last launch
+  int timed_jobs[kSlots] = {};           // jobs and class of each launch of the last plan
+  int timed_class[kSlots] = {};
   Pool pool;
   int sm_count = 0;
   int priority = 0;                        // of small launches (small_priority)
@@ -778,17 +781,18 @@ struct Plan {
   bool small = false;           // a launch of few CTAs: placed before a larger one's waiting CTAs
 };
 
-// The side stream and events of every slot the plan uses, made on the slot's
-// first use (planning, never launching: a launch may be captured).
-sfd_status ensure_slots(sfd_ctx* c, const Plan& P) {
-  for (int k = 0; k < kSlots; ++k) {
-    if (P.first[k + 1] == P.first[k] || c->join[k]) continue;
+// Side streams and events for a plan of n launches.  A context starts with
+// kClasses of them and planning adds what a larger plan needs (never the
+// launch, which may be captured), so that a first call makes none.
+sfd_status ensure_lanes(sfd_ctx* c, int n) {
+  for (int q = 0; q < n; ++q) {
+    if (c->join[q]) continue;
     cudaEvent_t j = nullptr;
-    if (!c->side[k]) SFD_CUDA(cudaStreamCreateWithFlags(&c->side[k], cudaStreamNonBlocking));
-    if (!c->t0[k]) SFD_CUDA(cudaEventCreate(&c->t0[k]));
-    if (!c->t1[k]) SFD_CUDA(cudaEventCreate(&c->t1[k]));
+    if (!c->side[q]) SFD_CUDA(cudaStreamCreateWithFlags(&c->side[q], cudaStreamNonBlocking));
+    if (!c->t0[q]) SFD_CUDA(cudaEventCreate(&c->t0[q]));
+    if (!c->t1[q]) SFD_CUDA(cudaEventCreate(&c->t1[q]));
     SFD_CUDA(cudaEventCreateWithFlags(&j, cudaEventDisableTiming));
-    c->join[k] = j;
+    c->join[q] = j;
   }
   return SFD_OK;
 }
@@ -987,7 +991,9 @@ sfd_status make_plan(sfd_ctx* c, const std::vector<Job>& jobs, const std::vector
     std::stable_sort(P.order, P.order + kSlots, [&](int x, int y) { return share(x) > share(y); });
   }
   P.small = n_ctas <= sms / 2;
-  return ensure_slots(c, P);
+  int launches = 0;
+  for (int k = 0; k < kSlots; ++k) launches += P.first[k + 1] > P.first[k];
+  return ensure_lanes(c, launches);
 }
 
 // Launch priority of small plans on `stream` (0: none): one above a stream's
@@ -1015,30 +1021,32 @@ sfd_status issue_plan(sfd_ctx* c, const Plan& P, const Job* d_jobs) {
   for (int k = 0; k < kSlots; ++k) active += P.first[k + 1] > P.first[k];
   if (active == 0) return SFD_OK;
   if (active > 1) SFD_CUDA(cudaEventRecord(c->fork, c->stream));
-  for (int k = 0; k < kSlots; ++k) c->timed_jobs[k] = 0;
-  for (int kk = 0; kk < kSlots; ++kk) {
+  for (int q = 0; q < kSlots; ++q) c->timed_jobs[q] = 0;
+  for (int kk = 0, q = 0; kk < kSlots; ++kk) {   // (q: the launch's place)
     const int k = P.order[kk];
     const int n_k = P.first[k + 1] - P.first[k];
     if (n_k == 0) continue;
     cudaStream_t st = c->stream;
     if (active > 1) {
-      st = c->side[k];
+      st = c->side[q];
       SFD_CUDA(cudaStreamWaitEvent(st, c->fork, 0));
     }
-    if (c->timing) SFD_CUDA(cudaEventRecord(c->t0[k], st));
+    if (c->timing) SFD_CUDA(cudaEventRecord(c->t0[q], st));
     cudaError_t e = kLaunch[k % kClasses](d_jobs + P.first[k], n_k, c->d_counter + k * c->sm_count, P.wf[k],
                                P.regions[k] * P.group[k], P.ctas[k], P.queued[k], P.group[k], P.small ? c->priority : 0,
                                st);
     if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
     if (c->timing) {
-      SFD_CUDA(cudaEventRecord(c->t1[k], st));
-      c->timed_jobs[k] = n_k;
+      SFD_CUDA(cudaEventRecord(c->t1[q], st));
+      c->timed_jobs[q] = n_k;
+      c->timed_class[q] = k % kClasses;
     }
     c->last_launches++;
     if (active > 1) {
-      SFD_CUDA(cudaEventRecord(c->join[k], st));
-      SFD_CUDA(cudaStreamWaitEvent(c->stream, c->join[k], 0));
+      SFD_CUDA(cudaEventRecord(c->join[q], st));
+      SFD_CUDA(cudaStreamWaitEvent(c->stream, c->join[q], 0));
     }
+    ++q;
   }
   return SFD_OK;
 }
@@ -1090,10 +1098,10 @@ sfd_status copy_out_by_class(sfd_ctx* c, const Plan& P, const float* dout, float
   int active = 0;
   for (int k = 0; k < kSlots; ++k) active += P.first[k + 1] > P.first[k];
   const cudaStream_t st = active > 1 ? c->copy : c->stream;
-  for (int kk = 0; kk < kSlots; ++kk) {
+  for (int kk = 0, q = 0; kk < kSlots; ++kk) {
     const int k = P.order[kk];
     if (P.first[k + 1] == P.first[k]) continue;
-    if (active > 1) SFD_CUDA(cudaStreamWaitEvent(st, c->join[k], 0));
+    if (active > 1) SFD_CUDA(cudaStreamWaitEvent(st, c->join[q++], 0));
     for (int j = P.first[k]; j < P.first[k + 1]; ++j) {
       const Job& J = P.jobs[j];
       SFD_CUDA(d2h(c, out_host + (J.out - dout), J.out, sizeof(float) * static_cast<size_t>(J.n_samples), st));
@@ -1258,7 +1266,8 @@ sfd_status sfd_ctx_create(int device, void* cuda_stream, size_t mem_budget_bytes
   }
   bool ok = cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) == cudaSuccess &&
             cudaEventCreateWithFlags(&c->copied, cudaEventDisableTiming) == cudaSuccess &&
-            cudaStreamCreateWithFlags(&c->copy, cudaStreamNonBlocking) == cudaSuccess;
+            cudaStreamCreateWithFlags(&c->copy, cudaStreamNonBlocking) == cudaSuccess &&
+            ensure_lanes(c, kClasses) == SFD_OK;
   if (!ok) {
     sfd_ctx_destroy(c);
     return fail(SFD_ECUDA, "stream/event creation failed");
@@ -1344,13 +1353,14 @@ sfd_status sfd_ctx_kernel_times(sfd_ctx* c, float* ms, int32_t* n_jobs) {
   sfd_status rc = set_device(c);
   if (rc) return rc;
   for (int k = 0; k < kClasses; ++k) ms[k] = 0.f, n_jobs[k] = 0;
-  for (int k = 0; c->timing && k < kSlots; ++k) {   // a class's launches run side by side: the longer one
-    if (c->timed_jobs[k] == 0) continue;
+  for (int q = 0; c->timing && q < kSlots; ++q) {   // a class's launches run side by side: the longer one
+    if (c->timed_jobs[q] == 0) continue;
+    const int k = c->timed_class[q];
     float t = 0.f;
-    SFD_CUDA(cudaEventSynchronize(c->t1[k]));
-    SFD_CUDA(cudaEventElapsedTime(&t, c->t0[k], c->t1[k]));
-    ms[k % kClasses] = std::max(ms[k % kClasses], t);
-    n_jobs[k % kClasses] += c->timed_jobs[k];
+    SFD_CUDA(cudaEventSynchronize(c->t1[q]));
+    SFD_CUDA(cudaEventElapsedTime(&t, c->t0[q], c->t1[q]));
+    ms[k] = std::max(ms[k], t);
+    n_jobs[k] += c->timed_jobs[q];
   }
   return SFD_OK;
 }
