@@ -134,6 +134,11 @@ __global__ void __launch_bounds__(kThreads, 1) adjoint_rows_kernel(const AdjJob*
     wm[q] = w;
     w1m[q] = 1.0f - wm[q];
   }
+  // the row's weights in P^T, in double-floats as in sfd_adjoint.cu (wm, w1m
+  // are the forward's own floats; with those the gradients of plucked and
+  // bowed strings were up to 5e-6 from that kernel's, with these 2e-9)
+  dfl::NodeWeights wt = {1.0f, 0.0f};
+  if (has_z && act) wt = dfl::node_weights((i + 1) * n_l - mm[1] * n_t, n_t, 1.0f / static_cast<R>(n_t));
   if (has_z)
 #pragma unroll 1
     for (int m = tid; m <= n_l + 1; m += T) {   // n_z + 3 entries
@@ -295,12 +300,12 @@ __global__ void __launch_bounds__(kThreads, 1) adjoint_rows_kernel(const AdjJob*
       __syncthreads();
       if (act) {   // d_+[g d_- x] at the row, times the row's weights
         const R f = (get(X + i + 1) - x) * gr - (x - get(X + i - 1)) * gl;
-        put(P0 + i, w1m[1] * f);
-        put(P1 + i, wm[1] * f);
+        put(P0 + i, wt.left * f);
+        put(P1 + i, wt.right * f);
         if (two) {
           const R h = (get(XP + i + 1) - y) * gr - (y - get(XP + i - 1)) * gl;
-          put(Q0 + i, w1m[1] * h);
-          put(Q1 + i, wm[1] * h);
+          put(Q0 + i, wt.left * h);
+          put(Q1 + i, wt.right * h);
         }
       }
       __syncthreads();
@@ -568,8 +573,8 @@ __global__ void __launch_bounds__(kThreads, 1) adjoint_rows_kernel(const AdjJob*
       add(kGS1, xi * (2.0f * d2du + d2a), false);
       if (has_z) {
         const R f = get(P1 + i + 1) - get(P1 + i);   // d_+[psi g] at the row
-        put(Q0 + i, w1m[1] * f);
-        put(Q1 + i, wm[1] * f);
+        put(Q0 + i, wt.left * f);
+        put(Q1 + i, wt.right * f);
       }
     }
     if (has_z) {

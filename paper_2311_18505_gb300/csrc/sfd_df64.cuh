@@ -119,6 +119,20 @@ __device__ __forceinline__ df64 fabs(df64 a) { return a.hi < 0.f || (a.hi == 0.f
 __device__ __forceinline__ df64 fmax(df64 a, df64 b) { return a < b ? b : a; }
 __device__ __forceinline__ df64 fma(df64 a, df64 b, df64 c) { return a * b + c; }
 
+// Weights of P^T at a transverse node `rem` n_t-ths into a longitudinal
+// interval (0 <= rem < n_t), on the interval's two nodes: 1 - rem / n_t and
+// rem / n_t, from exact integers, inv_nt = 1 / n_t.  (The forward's weights,
+// which the interpolation P uses in the adjoint too, are floats.)
+struct NodeWeights {
+  df64 left, right;
+};
+__device__ __forceinline__ NodeWeights node_weights(int rem, int n_t, df64 inv_nt) {
+  NodeWeights w;
+  w.left = 1.f - df64(rem) * inv_nt;
+  w.right = rem > 0 ? 1.f - df64(n_t - rem) * inv_nt : df64(0.f);
+  return w;
+}
+
 // conversions with FP64 (segment boundaries and the host-facing results only)
 __device__ __forceinline__ df64 df_from_double(double d) {
   const float h = static_cast<float>(d);
