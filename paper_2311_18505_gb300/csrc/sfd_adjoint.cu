@@ -627,6 +627,8 @@ cudaError_t raise_adjoint_smem_limit() {
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(adjoint_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            optin - static_cast<int>(fa.sharedSizeBytes));
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(adjoint_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, kSmemCarveout);
   if (e == cudaSuccess) g_adj_attr_done[dev] = true;
   return e;
 }

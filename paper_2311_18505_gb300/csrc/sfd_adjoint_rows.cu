@@ -693,6 +693,8 @@ cudaError_t launch_adjoint_rows(const AdjJob* d_jobs, int n_jobs, int threads, i
       e = cudaFuncSetAttribute(adjoint_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                optin - static_cast<int>(fixed));
       if (e != cudaSuccess) return e;
+      e = cudaFuncSetAttribute(adjoint_rows_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, kSmemCarveout);
+      if (e != cudaSuccess) return e;
       g_rows_done[dev] = true;
     }
   }

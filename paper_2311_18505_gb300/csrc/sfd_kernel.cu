@@ -184,15 +184,7 @@ cudaError_t raise_smem_limit() {
   e = cudaFuncSetAttribute(SFD_KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            optin - static_cast<int>(fa.sharedSizeBytes));
   if (e != cudaSuccess) return e;
-  // One division of an SM's L1 for the launches of all classes.  Left to the
-  // runtime it follows each launch's own need, and an SM that runs CTAs under
-  // one division starts none that want another until it is empty: with a
-  // group of 4 warps on every SM, half of its registers free, a one-note call
-  // of another context waited 39 ms for the first to end, now takes 0.3 (alone
-  // 0.2).  164 of 228 KB for shared memory: with all of it the spills of the
-  // widest instances miss what is left (96 kHz bass strings 8.25 -> 8.62 ms a
-  // block of 1024), with 164, 132 or the runtime's choice they take the same.
-  e = cudaFuncSetAttribute(SFD_KERNEL, cudaFuncAttributePreferredSharedMemoryCarveout, 72);
+  e = cudaFuncSetAttribute(SFD_KERNEL, cudaFuncAttributePreferredSharedMemoryCarveout, kSmemCarveout);
   if (e == cudaSuccess) g_attr_done[dev] = true;
   return e;
 }

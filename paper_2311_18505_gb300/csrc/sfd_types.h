@@ -138,6 +138,16 @@ constexpr int kMaxRegRows = 9;
 // static shared memory of the register-path kernels (the warp pairs'
 // exchange cells and job index cells); dynamic regions get the rest
 constexpr int kStaticSmemBytes = 2 * 1024 * 4 + 4 * 4;
+// Shared memory's part of an SM's L1 that every kernel prefers, in per cent
+// (164 of 228 KB).  Left to the runtime it follows each launch's own need, and
+// an SM that runs CTAs under one division starts none that want another until
+// it is empty: with a group of 4 warps on every SM, half of its registers
+// free, a one-note call of another context waited 39 ms for the first to end,
+// beside the reverse sweep of 152 strings 5.8 ms; now both take 0.3 (alone
+// 0.2).  With all of L1 for shared memory the spills of the widest step
+// instances miss what is left (96 kHz bass strings 8.25 -> 8.62 ms a block of
+// 1024); with 164, 132 KB or the runtime's choice they take the same.
+constexpr int kSmemCarveout = 72;
 constexpr int kArraysU = 19;
 constexpr int kArraysZ = 15;
 inline __host__ __device__ int warp_smem_floats(int m_u, int m_z, int z_jacobi) {

@@ -2,6 +2,7 @@
 batch that another context (on a stream of its own) is stepping, as long as
 the batch leaves warps free; its samples are those it has alone."""
 
+import threading
 import time
 
 import numpy as np
@@ -79,3 +80,46 @@ def test_a_call_beside_another_contexts_batch(batch, notes):
         assert best < 0.25 * t_big, (best, t_big)
     finally:
         big.close()
+
+
+def test_a_call_beside_another_contexts_tape():
+    """One note while another context's tape runs its reverse sweep on every SM
+    (blocks of 192 threads and 100 KB, which leave warps and memory free)."""
+    from paper_2311_18505_gb300 import sfd
+    n = 1024
+    dicts = [string(188, 280, "pluck")] * torch.cuda.get_device_properties(0).multi_processor_count
+    note = [string(100, 80, "bow")]
+    alone = Batch(sfd, note, NOTE)
+    alone.timed()
+    ref = alone.out.cpu().numpy()
+    alone.close()
+    stream = torch.cuda.Stream()
+    ctx = sfd.sfd_ctx_create(0, stream.cuda_stream, 256 << 20)
+    tape = sfd.sfd_tape_create(ctx, dicts, n, n)
+    try:
+        with torch.cuda.stream(stream):
+            y = torch.empty(len(dicts), n, device="cuda")
+            w = torch.ones(len(dicts), n, device="cuda")
+        torch.cuda.synchronize()
+        sfd.sfd_tape_forward(tape, y)
+        backward = lambda: sfd.sfd_tape_backward(tape, w, len(dicts))
+        backward()
+        t = time.perf_counter()
+        backward()
+        t_back = time.perf_counter() - t
+        best = float("inf")
+        for _ in range(3):
+            call = Batch(sfd, note, NOTE)
+            thread = threading.Thread(target=backward)
+            thread.start()
+            time.sleep(0.3 * t_back)
+            best = min(best, call.timed())
+            running = thread.is_alive()
+            thread.join()
+            assert np.array_equal(call.out.cpu().numpy(), ref)
+            call.close()
+            assert running or best > 0.5 * t_back
+        assert best < 0.25 * t_back, (best, t_back)
+    finally:
+        sfd.sfd_tape_destroy(tape)
+        sfd.sfd_ctx_destroy(ctx)
