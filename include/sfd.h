@@ -32,6 +32,10 @@
  *
  * Threading.  Objects are not thread-safe; distinct contexts may be used
  * from distinct threads.  Calls on one context are ordered on its stream.
+ * Contexts on streams of their own run side by side on one GPU: a batch leaves
+ * what its strings do not need, and the kernels of a call that needs at most
+ * half of the SMs are launched one priority above a stream's default, so that
+ * they start before the waiting blocks of a larger batch.
  */
 #ifndef SFD_H
 #define SFD_H

@@ -303,17 +303,13 @@ struct WarpGroup {
 };
 
 // One job of one string that is not unstable yet.  MZ: longitudinal rows per
-// lane held in registers (0: no longitudinal grid; 1 or 3, folded into the sweeps, one warp; 403, 803:
-// up to 12 or 24, three in the registers of each of a group's 4 or 8 warps), -1 for
-// any number kept in shared memory (folded, warp groups), -2 for a factored
-// longitudinal matrix (shared memory, one warp).
+// lane held in registers (0: no longitudinal grid; 1 or 3, folded into the
+// sweeps, one warp; 403, 803: up to 12 or 24, three in the registers of each
+// of a group's 4 or 8 warps), -1 for any number kept in shared memory (folded,
+// one warp or a group), -2 for a factored longitudinal matrix (shared memory,
+// one warp).
 // Not inlined: each instance gets its own registers (inlined side by side in
 // one kernel, the descriptor loads of all of them were hoisted together).
-// A step is one dependent chain, bound by the latency of its operations and
-// by instruction fetch, so an instance holds only what its strings execute:
-// plucked, one row per lane 3.0 us a step with one loop for every kind, 1.9
-// so; three rows 3.0 and 1.9; five 4.8 and 2.5; bowed 3.9 and 2.85, 4.05 and
-// 2.65, 6.1 and 3.35; linear 1.04 and 0.41 (one string alone).
 // The region is passed as an offset into the CTA's shared memory, so that
 // the accesses stay shared-memory instructions.
 template <int MU, int MZ, int EXC, bool LIN>

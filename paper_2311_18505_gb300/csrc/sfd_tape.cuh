@@ -156,8 +156,13 @@ sfd_status sfd_tape_create(sfd_ctx* c, int32_t n, const sfd_string_params* param
   }
   // Which adjoint kernel: one thread per row wherever the grid allows it (at
   // most 255 transverse rows, longitudinal off-diagonal folded into the
-  // sweeps: its chain is shorter at every size: 20 us a step against 41 on 64 strings
-  // of 40-1000 Hz, 15 against 26 on one of 31 x 4 rows); larger or strongly damped grids take four warps per string.
+  // sweeps): its chain is shorter at every size, 20 us a step against 41 on 64
+  // strings of 40-1000 Hz, 15 against 26 on one of 31 x 4 rows.  It also holds
+  // where a tape has more strings than the GPU has SMs, although one block
+  // then fills an SM that holds two of the other kernel's: reverse sweeps of 240
+  // samples, 304 strings of up to 152 x 374 rows 13.3 ms against 23.4, 608 of
+  // them 23.2 against 45.8, 1216 of up to 49 x 70 rows 14.7 against 52.3.
+  // Larger or strongly damped grids take four warps per string.
   if (rc == SFD_OK) {
     std::vector<int> rest;
     for (int i = 0; i < n; ++i) {

@@ -135,7 +135,7 @@ struct AdjJob {
 // Up to kMaxRegRows transverse rows per lane live in registers (2 transverse
 // transfer arrays in shared memory); larger grids use the shared-memory path.
 constexpr int kMaxRegRows = 9;
-// static shared memory of the register-path kernels (the warp pairs'
+// static shared memory of the register-path kernels (the warp groups'
 // exchange cells and job index cells); dynamic regions get the rest
 constexpr int kStaticSmemBytes = 2 * 1024 * 4 + 4 * 4;
 // Shared memory's part of an SM's L1 that every kernel prefers, in per cent
