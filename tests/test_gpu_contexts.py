@@ -68,15 +68,17 @@ def test_a_call_beside_another_contexts_batch(batch, notes):
         big.timed()
         t_big = big.timed()
         best = float("inf")
-        for _ in range(3):   # (a stream may share a hardware queue with one of the batch's: the best of three)
+        # (a stream may share a hardware queue with one of the batch's, and the
+        # host may be late: the best of the tries that met the batch running)
+        for _ in range(5):
             call = Batch(sfd, dicts, NOTE)
             big.launch()
             time.sleep(0.1 * t_big)
-            best = min(best, call.timed())
-            running = not big.stream.query()
+            t = call.timed()
+            if not big.stream.query():
+                best = min(best, t)
             assert np.array_equal(call.out.cpu().numpy(), ref)
             call.close()
-            assert running or best > 0.5 * t_big
         assert best < 0.25 * t_big, (best, t_big)
     finally:
         big.close()
@@ -108,17 +110,17 @@ def test_a_call_beside_another_contexts_tape():
         backward()
         t_back = time.perf_counter() - t
         best = float("inf")
-        for _ in range(3):
+        for _ in range(5):
             call = Batch(sfd, note, NOTE)
             thread = threading.Thread(target=backward)
             thread.start()
             time.sleep(0.3 * t_back)
-            best = min(best, call.timed())
-            running = thread.is_alive()
+            t = call.timed()
+            if thread.is_alive():
+                best = min(best, t)
             thread.join()
             assert np.array_equal(call.out.cpu().numpy(), ref)
             call.close()
-            assert running or best > 0.5 * t_back
         assert best < 0.25 * t_back, (best, t_back)
     finally:
         sfd.sfd_tape_destroy(tape)
